@@ -15,6 +15,10 @@ struct Tab {
   T D[MAXN][MAXN];      // GLL Lagrange derivatives at Gauss points
   T Dc[MAXN][MAXN];     // collocation derivative at Gauss points Dc[q][p]
   T Dend[2][MAXN];      // GLL Lagrange derivatives at x = 0, 1
+  // odd n = r + 2, H = n / 2: the tables of B and Dc on the even (e) and odd (o) parts of a line,
+  // Xe, Xo[q][j] = (X[q][j] +- X[q][n-1-j]) / 2, their middle columns Xm[q] = X[q][H] and the middle
+  // row Dh[j] = Dc[H][j]
+  T Be[2][2], Bo[2][2], Bm[2], De[2][2], Do[2][2], Dm[2], Dh[2];
   T P1[MAXN][4];        // Legendre P_i(2x-1) at Gauss points
   T Pend[2][4];         // Legendre at x = 0, 1
   T qx[MAXN], qw[MAXN], gll[MAXN];
@@ -78,6 +82,19 @@ Tab<T> make_tab(const LevelTables& L, double tau) {
     for (int j = 0; j < MAXN; ++j) {
       t.B[i][j] = (T)L.B[i][j]; t.D[i][j] = (T)L.D[i][j]; t.Dc[i][j] = (T)L.Dc[i][j];
     }
+  const int n = L.r + 2, H = n / 2;
+  if (n % 2 == 1)
+    for (int q = 0; q < H; ++q) {
+      for (int j = 0; j < H; ++j) {
+        t.Be[q][j] = (T)(0.5 * (L.B[q][j] + L.B[q][n - 1 - j]));
+        t.Bo[q][j] = (T)(0.5 * (L.B[q][j] - L.B[q][n - 1 - j]));
+        t.De[q][j] = (T)(0.5 * (L.Dc[q][j] + L.Dc[q][n - 1 - j]));
+        t.Do[q][j] = (T)(0.5 * (L.Dc[q][j] - L.Dc[q][n - 1 - j]));
+      }
+      t.Bm[q] = (T)L.B[q][H];
+      t.Dm[q] = (T)L.Dc[q][H];
+      t.Dh[q] = (T)L.Dc[H][q];
+    }
   for (int s = 0; s < 2; ++s) {
     for (int j = 0; j < MAXN; ++j) t.Dend[s][j] = (T)L.Dend[s][j];
     for (int i = 0; i < 4; ++i) t.Pend[s][i] = (T)L.Pend[s][i];
@@ -122,6 +139,7 @@ struct LevelArgs {
 };
 
 constexpr int kProblemUser = 5;   // STMG_USER
+constexpr int kProblemMms2d = 1, kProblemMms3d = 3;   // STMG_MMS2D, STMG_MMS3D: the data sets with a body force
 
 // Index of the boundary face (axis, side) of cell cc among the n^(D-1) faces of that side.
 template <int D>

@@ -18,14 +18,14 @@ struct Level {
   double* verts64 = nullptr;          // device, (n+1)^d * d
   float* verts32 = nullptr;
   ColorInfo colors[8]{};
-  int* bcells[8]{};                   // device lists of boundary cells per colour
-  int nbcells[8]{};
   int ncolors = 0;
   double hscale = 0;                  // Nitsche length factor (see LevelArgs)
   int64_t chunk_cells = 262144;       // cells per chunk of the smoother build's element scratch
   int smoother = 0;                   // 0: surrogate patches (Sec. 4.3); 1: diagonal space-time Vanka
   double* geo64 = nullptr;            // 2D: geometry table of the Jacobian apply (see OpArgs::geo)
   float* geo32 = nullptr;
+  void* cellbuf = nullptr;            // cell-wise results of the operator kernels (CellBuf), one buffer
+  size_t cellbuf_bytes = 0;           // for all levels of a handle, on the handle's stream only
 };
 
 struct Problem {
@@ -52,12 +52,25 @@ cudaError_t launch_operator(const Level& lv, const Problem& pb, int mode, double
                             int batch = 1, int64_t xs = 0, int64_t ys = 0);
 
 // y = rhs - J(state) x on a level (rhs null: y = J(state) x), the residual of a multigrid sweep;
-// one launch where the tiled 2D kernel applies, else the operator followed by a vector update.
+// one launch where the tiled 2D kernel applies, else the cell kernel and the node sums.
 // `columns` independent residuals at strides n_st (own rhs, x, state, y; per-column viscosity
 // nub[column] on the device, or null for pb.nu).
 template <typename T>
 cudaError_t launch_level_residual(const Level& lv, const Problem& pb, const T* rhs, const T* x, const T* state, T* y,
                                   cudaStream_t stream, int columns = 1, const T* nub = nullptr);
+
+// Bytes of the cell buffer that the operator calls of a level use at most: one column of cell-wise FP64
+// results, capped at 1 GiB (larger meshes run in chunks of cell planes; two planes at least), and
+// at least 16 MiB, so that the batched applies of small levels share launches.
+inline size_t cellbuf_need(int d, int n, int r, int k) {
+  double plane = 8.0 * (k + 1) * d, cells = 1;
+  for (int l = 0; l < d; ++l) plane *= r + 2;
+  for (int l = 0; l + 1 < d; ++l) cells *= n;
+  plane *= cells;
+  double b = plane * n;
+  if (b > 1073741824.0) b = plane * 2 > 1073741824.0 ? plane * 2 : 1073741824.0;
+  return (size_t)(b < 16777216.0 ? 16777216.0 : b);
+}
 
 cudaError_t launch_initial_condition(const Level& lv, const Problem& pb, double* V0, cudaStream_t s);
 

@@ -1,7 +1,6 @@
 // FP32 operator kernels: the Jacobian apply used on the levels of the multigrid preconditioner.
 #include <type_traits>
 #include "op_launch.cuh"
-#include "vec.cuh"
 
 namespace stmg {
 
@@ -22,9 +21,7 @@ cudaError_t launch_level_residual<float>(const Level& lv, const Problem& pb, con
                                        const float* state, float* y, cudaStream_t s, int columns, const float* nub) {
   cudaError_t e = launch_jac_tiled<float>(lv, pb, x, state, rhs, y, s, columns, nub);
   if (e != cudaErrorNotSupported) return e;
-  e = launch_any<float, MJ>(lv, pb, 0.0, x, state, nullptr, y, s, columns, lv.Nst, lv.Nst, lv.Nst, nub);
-  if (e == cudaSuccess && rhs) e = vaxpby<float>(columns * lv.Nst, 1.0f, rhs, -1.0f, y, s);
-  return e;
+  return launch_any<float, MJ>(lv, pb, 0.0, x, state, nullptr, y, s, columns, lv.Nst, lv.Nst, lv.Nst, nub, rhs);
 }
 
 }  // namespace stmg

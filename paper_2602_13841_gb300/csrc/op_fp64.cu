@@ -2,7 +2,6 @@
 // nodal interpolation of the initial velocity.
 #include <type_traits>
 #include "op_launch.cuh"
-#include "vec.cuh"
 
 namespace stmg {
 
@@ -20,9 +19,7 @@ cudaError_t launch_level_residual<double>(const Level& lv, const Problem& pb, co
                                        const double* state, double* y, cudaStream_t s, int columns, const double* nub) {
   cudaError_t e = launch_jac_tiled<double>(lv, pb, x, state, rhs, y, s, columns, nub);
   if (e != cudaErrorNotSupported) return e;
-  e = launch_any<double, MJ>(lv, pb, 0.0, x, state, nullptr, y, s, columns, lv.Nst, lv.Nst, lv.Nst, nub);
-  if (e == cudaSuccess && rhs) e = vaxpby<double>(columns * lv.Nst, 1.0, rhs, -1.0, y, s);
-  return e;
+  return launch_any<double, MJ>(lv, pb, 0.0, x, state, nullptr, y, s, columns, lv.Nst, lv.Nst, lv.Nst, nub, rhs);
 }
 
 // v_{0,h}: v0 evaluated at the mapped Gauss-Lobatto nodes (one thread per global node).

@@ -3,7 +3,7 @@
 #include <type_traits>
 #include "level.hpp"
 #include "operator.cuh"
-#include "operator2d.cuh"
+#include "operator_cells.cuh"
 #include "operator2d_tile.cuh"
 #include "counters.hpp"
 #include <cstdlib>
@@ -25,76 +25,83 @@ LevelArgs<T> level_args(const Level& lv, const Problem& pb, double t0) {
   return a;
 }
 
-template <typename T, int D, int N, int MODE>
-static int vol_smem_per_cell(int kp1) {
-  constexpr int Q = Shape<D, N>::Q;
-  return ((MODE == MJ ? 3 : 2) * kp1 * D * Q + D * D * Q + 2 * D * Q + Q + kp1 * MAXNP + 8 * 3) * (int)sizeof(T);
+// Cells per block of the cell kernels: the count whose threads fill whole warps best (the FP64 pipe
+// is paid for by the warp), the largest among equals; fewer on meshes that would not give every SM
+// two blocks.
+inline int cells_per_block(int threads_per_cell, int max_threads, int64_t cells) {
+  int best = 1;
+  double eff = 0.0;
+  for (int c = 1; c * threads_per_cell <= max_threads; ++c) {
+    const int t = c * threads_per_cell;
+    const double e = (double)t / ((t + 31) / 32 * 32);
+    if (e >= eff) { eff = e; best = c; }
+  }
+  const int64_t spread = (cells + 303) / 304;
+  return spread < best ? (int)spread : best;
 }
 
-template <typename T, int D, int N>
-static int face_smem_per_cell(int kp1) {
-  constexpr int Q = Shape<D, N>::Q;
-  constexpr int NF = Shape<D, N>::NF;
-  return (2 * kp1 * D * Q + kp1 * MAXNP + D * NF + D * D * NF + NF + Q + 4 + 8 * 3) * (int)sizeof(T);
-}
-
+// One operator call in two launches per chunk (cells, node sums): whole columns while they fit the
+// level's cell buffer, else one column at a time in chunks of cell planes.
 template <typename T, int D, int N, int MODE>
 static cudaError_t launch_dn(const Level& lv, const Problem& pb, double t0, const T* x,
                              const T* state, const T* vprev, T* y, cudaStream_t stream,
-                             int batch, int64_t xs, int64_t ys, int64_t ss = 0, const T* nub = nullptr) {
-  constexpr int Q = Shape<D, N>::Q;
+                             int batch, int64_t xs, int64_t ys, int64_t ss, const T* nub, const T* rhs) {
+  constexpr int TPG = D == 2 ? N : N * N;             // threads per (cell, time node)
+  constexpr bool F64 = sizeof(T) == 8;
+  constexpr int BT = D == 3 && (N == 5 || !F64) ? 256 : 192;
+  constexpr int MINB = D == 2 ? (F64 ? 2 : 4) : (F64 && N == 5 ? 1 : 2);
   const int kp1 = lv.k + 1;
-  Tab<T> tb = make_tab<T>(lv.tabs, pb.tau);
+  const Tab<T> tb = make_tab<T>(lv.tabs, pb.tau);
   const T* geo = nullptr;
   if constexpr (D == 2) {
-    if constexpr (std::is_same<T, double>::value) geo = lv.geo64; else geo = lv.geo32;
+    if constexpr (F64) geo = lv.geo64; else geo = lv.geo32;
   }
-  OpArgs<T> A{level_args<T>(lv, pb, t0), x, state, vprev, y, xs, ys, geo, ss, nub};
-  int cpb = 256 / Q; if (cpb < 1) cpb = 1;
-  int smem = cpb * vol_smem_per_cell<T, D, N, MODE>(kp1);
-  while (smem > 160 * 1024 && cpb > 1) { --cpb; smem = cpb * vol_smem_per_cell<T, D, N, MODE>(kp1); }
-  cudaError_t e = allow_smem(k_volume<T, D, N, MODE>, (size_t)smem);
-  if (e != cudaSuccess) return e;
-  // faces: one boundary cell per block, so that the loop over the six faces skips the faces the
-  // cell does not have (a block of several cells runs every face any of them has)
-  int fcpb = 1;
-  int fsmem = fcpb * face_smem_per_cell<T, D, N>(kp1);
-  while (fsmem > 160 * 1024 && fcpb > 1) { --fcpb; fsmem = fcpb * face_smem_per_cell<T, D, N>(kp1); }
-  if (MODE != MM) {
-    e = allow_smem(k_faces<T, D, N, MODE>, (size_t)fsmem);
-    if (e != cudaSuccess) return e;
-  }
-  for (int b = 0; b < batch; ++b) {
-    e = cudaMemsetAsync(y + b * ys, 0, sizeof(T) * lv.Nst, stream);
-    if (e != cudaSuccess) return e;
-  }
-  for (int c = 0; c < lv.ncolors; ++c) {
-    const ColorInfo& ci = lv.colors[c];
-    if (ci.count > 0) {
-      if constexpr (D == 2) {
-        // one group of Q lanes per (cell, time node)
-        constexpr int cpw = 32 / Q, per_block = 8 * cpw;
-        const int64_t groups = (int64_t)ci.count * kp1;
-        dim3 grid((unsigned)((groups + per_block - 1) / per_block), batch);
-        k_volume2d<T, N, MODE><<<grid, 256, 0, stream>>>(A, tb, ci);
-      } else {
-        dim3 grid((ci.count + cpb - 1) / cpb, batch);
-        k_volume<T, D, N, MODE><<<grid, cpb * Q, smem, stream>>>(A, tb, ci, cpb);
+  const int64_t cplane = D == 2 ? lv.n : (int64_t)lv.n * lv.n;   // cells per plane of the last axis
+  CellBuf<T> cb{};
+  cb.s = (T*)lv.cellbuf;
+  cb.plane = cplane * Shape<D, N>::Q;
+  const int64_t cap = (int64_t)(lv.cellbuf_bytes / sizeof(T)), per = (int64_t)kp1 * D * cb.plane;
+  const bool whole = per * lv.n <= cap;
+  cb.P = whole ? lv.n : (int)(cap / per);
+  if (!cb.s || cb.P < 2) { if (!(whole && cb.s)) return cudaErrorInvalidValue; }
+  cb.comp = cb.plane * cb.P;
+  cb.col = cb.comp * kp1 * D;
+  int64_t cols = whole ? cap / cb.col : 1;
+  if (cols > batch) cols = batch;
+  if (cols > 32768) cols = 32768;
+  const int step = whole ? lv.n : cb.P - 1;
+  auto kern = [] {
+    if constexpr (D == 2) return k_cells2d<T, N, MODE, BT, MINB>; else return k_cells3d<T, N, MODE, BT, MINB>;
+  }();
+  for (int64_t b0 = 0; b0 < batch; b0 += cols) {
+    const int nb = (int)(batch - b0 < cols ? batch - b0 : cols);
+    OpArgs<T> A{level_args<T>(lv, pb, t0), x + b0 * xs, state ? state + b0 * ss : nullptr, vprev, y + b0 * ys,
+                xs, ys, geo, ss, nub ? nub + b0 : nullptr};
+    const T* rb = rhs ? rhs + b0 * ys : nullptr;
+    for (int z0 = 0; z0 < lv.n; z0 += step) {
+      const int z1 = z0 + step < lv.n ? z0 + step : lv.n;
+      const int64_t c0 = z0 * cplane, c1 = z1 * cplane;
+      const int cpb = cells_per_block(TPG * kp1, BT, (c1 - c0) * nb);
+      const size_t smem = D == 2 ? cells2d_smem<T, N>(cpb, kp1) : cells3d_smem<T, N, MODE>(cpb, kp1);
+      if (smem > 48 * 1024) {
+        cudaError_t e = allow_smem(kern, smem);
+        if (e != cudaSuccess) return e;
       }
-      note_launch();
-    }
-    if (D == 3 && MODE != MM && lv.nbcells[c] > 0) {       // 2D: faces fused into k_volume2d
-      // one block per (boundary cell, time node) when fcpb == 1
-      dim3 grid(fcpb == 1 ? lv.nbcells[c] * kp1 : (lv.nbcells[c] + fcpb - 1) / fcpb, batch);
-      k_faces<T, D, N, MODE><<<grid, fcpb * Q, fsmem, stream>>>(A, tb, lv.bcells[c], lv.nbcells[c], fcpb);
-      note_launch();
+      const int threads = (cpb * kp1 * TPG + 31) / 32 * 32;
+      kern<<<dim3((unsigned)((c1 - c0 + cpb - 1) / cpb), nb), threads, smem, stream>>>(A, tb, cb, c0, c1, cpb, rb);
+      const int g0 = z0 * (N - 1), g1 = z1 == lv.n ? lv.N1 : z1 * (N - 1);
+      const int64_t nodes = (int64_t)(g1 - g0) * (D == 2 ? (int64_t)lv.N1 : (int64_t)lv.N1 * lv.N1);
+      const int64_t blocks = (nodes + 127) / 128;
+      k_node_sum<T, D, N><<<dim3((unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), nb), 128, 0, stream>>>(
+          cb, rb, A.y, lv.n, lv.N1, lv.nnodes, lv.Nv, kp1, ys, g0, nodes);
+      note_launch(2);
     }
   }
   return cudaGetLastError();
 }
 
-// Process-wide choice of the 2D Jacobian-apply kernel: the tiled single-launch kernel where it
-// applies (default), or the colour-split warp kernel when the environment variable STMG_APPLY2D
+// Process-wide choice of the 2D FP32 Jacobian-apply kernel: the tiled single-launch kernel where it
+// applies (default), or the cell kernel with node sums when the environment variable STMG_APPLY2D
 // is "colour" (kept for comparisons; read once).
 inline bool apply2d_tiled() {
   static const bool on = [] {
@@ -120,7 +127,7 @@ static cudaError_t jac_tiled_n(const Level& lv, const Problem& pb, const T* x, c
 // y = J(state) x, or y = rhs - J(state) x when rhs is not null, by the tiled 2D kernel (one
 // launch, y written without a zero fill).  `columns` independent applies at strides n_st (own
 // increment, state, output and, with nub, viscosity).  cudaErrorNotSupported where it does not
-// apply (3D, Q4/P3, FP64, or the colour kernels chosen).
+// apply (3D, Q4/P3, FP64, or the cell kernels chosen).
 template <typename T>
 cudaError_t launch_jac_tiled(const Level& lv, const Problem& pb, const T* x, const T* state, const T* rhs, T* y,
                              cudaStream_t s, int columns = 1, const T* nub = nullptr) {
@@ -137,9 +144,10 @@ cudaError_t launch_jac_tiled(const Level& lv, const Problem& pb, const T* x, con
 template <typename T, int MODE>
 static cudaError_t launch_any(const Level& lv, const Problem& pb, double t0, const T* x,
                               const T* state, const T* vprev, T* y, cudaStream_t s,
-                              int batch, int64_t xs, int64_t ys, int64_t ss = 0, const T* nub = nullptr) {
+                              int batch, int64_t xs, int64_t ys, int64_t ss = 0, const T* nub = nullptr,
+                              const T* rhs = nullptr) {
   const int N = lv.r + 2;
-#define STMG_LAUNCH(DD, NN) return launch_dn<T, DD, NN, MODE>(lv, pb, t0, x, state, vprev, y, s, batch, xs, ys, ss, nub)
+#define STMG_LAUNCH(DD, NN) return launch_dn<T, DD, NN, MODE>(lv, pb, t0, x, state, vprev, y, s, batch, xs, ys, ss, nub, rhs)
   if (lv.d == 2) {
     if (N == 3) STMG_LAUNCH(2, 3);
     if (N == 4) STMG_LAUNCH(2, 4);

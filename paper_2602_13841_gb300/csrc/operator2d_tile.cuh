@@ -1,7 +1,7 @@
 // Tiled 2D Jacobian apply: y = J_n(U) x, or y = rhs - J_n(U) x (the level residual of a
 // multigrid sweep), in one launch per apply.
 //
-// Same discrete operator as k_volume2d / k_faces (Sec. 4.4, Eq. JacobianLocal0-1): per cell and
+// Same discrete operator as k_cells2d (Sec. 4.4, Eq. JacobianLocal0-1): per cell and
 // time node a, the increment, the state and the time-mixed increment u_a = sum_b K_ab x_b are
 // interpolated to the Gauss points by two 1D passes, reference gradients are taken by the
 // collocation derivative, the flux of the linearised convection, viscosity and pressure is
@@ -19,7 +19,7 @@
 // classes of the cells one after another), so y is written once, with plain coalesced stores,
 // without atomics and without a zero fill: the result is deterministic.
 #pragma once
-#include "operator.cuh"
+#include "operator_cells.cuh"
 
 namespace stmg {
 

@@ -99,20 +99,6 @@ static void build_level(Handle* h, Level& lv, const std::vector<double>& verts) 
       ci.cnt[l] = (lv.n - bit + 1) / 2;
       ci.count *= ci.cnt[l];
     }
-    std::vector<int> bc;
-    for (int64_t cell = 0; cell < ncells; ++cell) {
-      int64_t rem = cell;
-      bool bnd = false, match = true;
-      for (int l = 0; l < lv.d; ++l) {
-        int x = (int)(rem % lv.n); rem /= lv.n;
-        if (x == 0 || x == lv.n - 1) bnd = true;
-        if ((x & 1) != ((c >> l) & 1)) match = false;
-      }
-      if (bnd && match) bc.push_back((int)cell);
-    }
-    lv.nbcells[c] = (int)bc.size();
-    lv.bcells[c] = (int*)h->dalloc(bc.size() * sizeof(int));
-    h->upload(lv.bcells[c], bc.data(), bc.size() * sizeof(int));
   }
   if (lv.d == 2) {
     // geometry table of the 2D Jacobian apply (5 values per cell and Gauss point, both precisions)
@@ -172,7 +158,7 @@ stmg_status stmg_footprint(const stmg_params* p, uint64_t* bytes) {
   int nn = n, hl = 0;
   while (nn % 2 == 0 && nn / 2 >= 2 && (p->n_levels_h < 0 || hl < p->n_levels_h)) { nn /= 2; ++hl; lv.push_back({nn, r, k}); }
   const double es = p->precond_precision == STMG_FP32 ? 4.0 : 8.0;
-  double tot = 0, ea = 0, eb = 0, em = 0, nvmax = 0, wk = 0;
+  double tot = 0, ea = 0, eb = 0, em = 0, nvmax = 0, wk = 0, cbuf = 0;
   std::vector<double> nst(lv.size());
   for (size_t l = 0; l < lv.size(); ++l) {
     const int ln = lv[l][0], lr = lv[l][1], lk = lv[l][2];
@@ -180,7 +166,8 @@ stmg_status stmg_footprint(const stmg_params* p, uint64_t* bytes) {
     double npc = (d == 2) ? (lr + 1.0) * (lr + 2.0) / 2.0 : (lr + 1.0) * (lr + 2.0) * (lr + 3.0) / 6.0;
     double Nv = d * nodes, Np = cells * npc;
     nst[l] = (lk + 1.0) * (Nv + Np);
-    tot += 12.0 * std::pow(ln + 1.0, d) + 4.0 * cells;                  // vertices, boundary lists
+    tot += 12.0 * d * std::pow(ln + 1.0, d);                            // vertices
+    cbuf = std::max(cbuf, (double)cellbuf_need(d, ln, lr, lk));
     if (d == 2) tot += cells * 5.0 * (lr + 2.0) * (lr + 2.0) * 12.0;    // 2D geometry tables
     tot += 5.0 * nst[l] * es;                                            // level vectors
     if (l + 1 < lv.size()) {
@@ -218,7 +205,7 @@ stmg_status stmg_footprint(const stmg_params* p, uint64_t* bytes) {
       tot += 3.0 * std::max((lk + 1.0) * Nv, (lk + 1.0) * Np) * es;      // transfer scratch
     }
   }
-  tot += (ea + eb + em + nvmax) * es + wk;
+  tot += (ea + eb + em + nvmax) * es + wk + cbuf;                        // cbuf: cell-wise operator results
   const double Nc = nst.back(), Nb = Nc + lv.back()[2] + 1;
   tot += Nb * Nb * 16.0 + Nc * Nc * 8.0;                                 // coarse factors
   tot += (2.0 * p->gmres_restart + 1.0 + 9.0) * nst[0] * 8.0;           // Krylov basis, Newton vectors
@@ -297,6 +284,10 @@ stmg_status stmg_create(const stmg_params* p, const double* vertices, stmg_strea
       build_level(h.get(), lv, cv);
       h->levels.push_back(lv);
     }
+    size_t cbytes = 0;
+    for (const Level& lv : h->levels) cbytes = std::max(cbytes, cellbuf_need(lv.d, lv.n, lv.r, lv.k));
+    void* cbuf = h->dalloc(cbytes);
+    for (Level& lv : h->levels) { lv.cellbuf = cbuf; lv.cellbuf_bytes = cbytes; }
   } catch (const std::bad_alloc&) {
     return STMG_ERR_OOM;
   } catch (const CudaFailure&) {
