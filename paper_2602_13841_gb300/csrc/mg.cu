@@ -65,15 +65,15 @@ cudaError_t MG<T>::allocate(Handle* hh, int slots) {
     Nc = (int)c.Nst;
     Nb = Nc + c.k + 1;
     A64 = (double*)h->dalloc((size_t)B * Nb * Nb * sizeof(double));
-    ident = (double*)h->dalloc(((size_t)Nc * Nc + 2 * (size_t)Nc) * sizeof(double));
+    ident = (double*)h->dalloc(((size_t)Nb * Nb + 2 * (size_t)Nc) * sizeof(double));
     Ucs = (double*)h->dalloc((size_t)Nc * sizeof(double));
     cb = (double*)h->dalloc((size_t)B * Nb * sizeof(double));
     cx = (double*)h->dalloc((size_t)B * Nb * sizeof(double));
     cr = (double*)h->dalloc((size_t)B * Nb * sizeof(double));
     cw = (double*)h->dalloc((size_t)B * Nb * sizeof(double));
     Ainv = (double*)h->dalloc((size_t)B * Nb * Nb * sizeof(double));
-    gj_col = (double*)h->dalloc((size_t)Nb * sizeof(double));
-    gj_piv = (int*)h->dalloc((size_t)Nb * sizeof(int));
+    gj_panel = (double*)h->dalloc(coarse_panel_entries(Nb) * sizeof(double));
+    gj_piv = (int*)h->dalloc(2 * (size_t)Nb * sizeof(int));
   } catch (const std::bad_alloc&) {
     return cudaErrorMemoryAllocation;
   } catch (const CudaFailure& f) {
@@ -135,7 +135,7 @@ cudaError_t MG<T>::setup(const double* U64, int slot, const Problem* pbp) {
   // A64 now holds J (N x N, column-major); move into the bordered layout via `ident` as staging
   CKE(cudaMemcpyAsync(ident, A64s, (size_t)Nc * Nc * sizeof(double), cudaMemcpyDeviceToDevice, s));
   CKE(coarse_border(c, pb, ident, A64s, Nc, Nb, s));
-  CKE(coarse_invert(A64s, Ainv + (int64_t)slot * Nb * Nb, gj_col, gj_piv, Nb, status, s));
+  CKE(coarse_invert(A64s, Ainv + (int64_t)slot * Nb * Nb, ident, gj_panel, gj_piv, Nb, status, s));
   int st = 0;
   CKE(cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, s));
   CKE(cudaStreamSynchronize(s));

@@ -41,7 +41,7 @@ struct MG {
   double *A64 = nullptr, *Ucs = nullptr, *cb = nullptr, *cx = nullptr, *cr = nullptr, *cw = nullptr;
   double* ident = nullptr;
   double* Ainv = nullptr;
-  double* gj_col = nullptr;
+  double* gj_panel = nullptr;
   int* gj_piv = nullptr;
   bool built = false;
   bool smoothable = true;            // every smoothed level's element matrices fit on-chip memory
@@ -95,8 +95,10 @@ bool vanka_supported(const Level& lv, size_t esize);
 // Coarse solver helpers (coarse.cu)
 cudaError_t coarse_border(const Level& lv, const Problem& pb, const double* J, double* A, int N, int Nb,
                           cudaStream_t s);
-cudaError_t coarse_invert(const double* A, double* Ainv, double* col, int* piv, int Nb, int* status,
+// work: Nb^2 entries, panel: coarse_panel_entries(Nb), piv: 2 Nb
+cudaError_t coarse_invert(const double* A, double* Ainv, double* work, double* panel, int* piv, int Nb, int* status,
                           cudaStream_t s);
+size_t coarse_panel_entries(int Nb);
 // y_j = A_j x_j for j < slots (A_j = A + j n^2, x_j = x + j n, y_j = y + j n); column-major.
 cudaError_t gemv_cm(const double* A, int n, const double* x, double* y, cudaStream_t s, int slots = 1);
 

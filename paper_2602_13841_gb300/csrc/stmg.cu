@@ -193,21 +193,17 @@ stmg_status stmg_footprint(const stmg_params* p, uint64_t* bytes) {
       const double ec = cells <= cap ? cells : std::min(cells, std::max(3.0, std::floor(cap / plane)) * plane);
       ea = std::max(ea, ec * mv * mv * (p->smoother == 2 ? lk + 1.0 : 1.0));
       eb = std::max(eb, ec * npc * mv); em = std::max(em, ec * nl * nl);
-      // patches beyond shared memory are factorised in a global workspace of 304 block slots
-      const double pslot = 2.0 * msp * msp + mv * mv + nl * nl;
-      if (p->smoother != 1 && es * (pslot + 2.0 * msp) + 4.0 * msp + 16.0 > 227.0 * 1024.0)
-        wk = std::max(wk, 304.0 * pslot * es);
-      // element tables beyond shared memory (3D Q4/P3) use 304 slots of the same workspace
-      const double nf = std::pow(lr + 2.0, d - 1);
-      const double etab = nl * nl * d + nl * nl + nl + nl * d + d * nl + d * (nf * (2.0 + 2.0 * d) + 2.0 * nf * nl) + 32.0;
-      if (es * etab > 227.0 * 1024.0) wk = std::max(wk, 304.0 * etab * es);
+      // patch matrices and element tables beyond shared memory: slots of a global workspace
+      Level tl;
+      tl.d = d; tl.r = lr; tl.npc = (int)npc; tl.smoother = p->smoother;
+      wk = std::max(wk, (double)vanka_work_entries(tl, (size_t)es) * es);
       nvmax = std::max(nvmax, Nv);
       tot += 3.0 * std::max((lk + 1.0) * Nv, (lk + 1.0) * Np) * es;      // transfer scratch
     }
   }
   tot += (ea + eb + em + nvmax) * es + wk + cbuf;                        // cbuf: cell-wise operator results
   const double Nc = nst.back(), Nb = Nc + lv.back()[2] + 1;
-  tot += Nb * Nb * 16.0 + Nc * Nc * 8.0;                                 // coarse factors
+  tot += Nb * Nb * 24.0 + Nb * 144.0;                                    // coarse factors
   tot += (2.0 * p->gmres_restart + 1.0 + 9.0) * nst[0] * 8.0;           // Krylov basis, Newton vectors
   *bytes = (uint64_t)tot;
   return STMG_OK;

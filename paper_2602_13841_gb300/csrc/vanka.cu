@@ -61,7 +61,7 @@ size_t vanka_elem_cells(const Level& lv) {
 }
 
 size_t vanka_work_entries(const Level& lv, size_t es) {
-  const size_t pw = (lv.smoother == 1 || patch_onchip(lv, es)) ? 0 : (size_t)kWorkSlots * work_slot(lv);
+  const size_t pw = (lv.smoother == 1 || patch_onchip(lv, es)) ? 0 : (size_t)kWorkSlots * work_slot(lv, es);
   const size_t ew = elem_onchip(lv, es) ? 0 : (size_t)kWorkSlots * elem_table_any(lv);
   return pw > ew ? pw : ew;
 }

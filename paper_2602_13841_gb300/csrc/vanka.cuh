@@ -6,13 +6,14 @@
 //        A_K = nu A + H'(v*) + N^c'(v*) + N^{b,r}   (velocity x velocity, boundary faces included)
 //        B_K = B + G^p                                (pressure x velocity)
 //        M_K                                          (scalar velocity mass)
-//   3. k_patch: the patch matrix is the global submatrix on the DoFs of K (all velocity and
+//   3. k_patch_small / k_patch_blocked: the patch matrix is the global submatrix on the DoFs of K (all velocity and
 //      pressure DoFs of K at all k+1 time nodes), so the velocity blocks sum the element
 //      matrices of every neighbour cell sharing both DoFs:
 //        S~_K = [ K^tau (x) M_patch + M^tau (x) A_patch ,  M^tau (x) B_K^T ]
 //               [ M^tau (x) B_K                         ,  0               ]
-//      M^tau = diag(w_a).  S~_K is inverted in shared memory by Gauss-Jordan elimination with
-//      partial pivoting; the inverse is stored column-major per cell.
+//      M^tau = diag(w_a).  S~_K is inverted through its time diagonalisation, one spatial system per
+//      eigenvalue, by Gauss-Jordan elimination with partial pivoting (vanka_patch.cuh); the inverse is
+//      stored column-major per cell.
 // Sweep (additive, damped): d <- d + omega sum_K R_K^T S~_K^{-1} R_K (rhs - J d); cells are
 // updated in 2^d colours so that the scatter is race free and deterministic.
 #pragma once
@@ -37,7 +38,7 @@ struct VankaArgs {
   __half* invh;         // the same scaled to [-1, 1] in FP16 with one FP32 factor per block
   float* scale;         // [cells][nblk]
   int* status;          // set to 1 on a zero pivot
-  T* work;              // global workspace of k_patch_global (null for on-chip patches) ...
+  T* work;              // global workspace of k_patch_blocked (null for on-chip patches) ...
   int64_t wslot;        // ... entries per block slot
 };
 
@@ -48,6 +49,13 @@ __host__ __device__ constexpr inline int inv_stride(int m, int es) {
   int st = m;
   while (((long long)m * st * es) % 16 != 0) ++st;
   return st;
+}
+
+// Rows of the spatial Vanka patch of Q_{N-1} / P_{N-2}^disc: D N^D velocity DoFs and C(r+D, D)
+// pressure modes (r = N - 2), known at compile time so that the row products unroll.
+template <int D, int N>
+__host__ __device__ constexpr int patch_rows() {
+  return D * Shape<D, N>::Q + (D == 2 ? (N - 1) * N / 2 : (N - 1) * N * (N + 1) / 6);
 }
 
 // max |x| over the block (all threads receive it)
@@ -94,9 +102,11 @@ __device__ void elem_cell(const VankaArgs<T>& V, const Tab<T>& tb, int64_t cell,
   T* s_v = s_jxw + Q;                    // [Q][D] v* at quadrature points
   T* s_vn = s_v + Q * D;                 // [D][NL] v* nodal
   T* s_f = s_vn + D * NL;                // per face: [NF] jxw, [NF][D] n, [NF] y, [NF][D] v, [NF][NL] phi, [NF][NL] dn
-  constexpr int FSZ = NF * (2 + 2 * D) + 2 * NF * NL;
+  constexpr int NP = patch_rows<D, N>() - MV;
+  constexpr int FSZ = NF * (2 + 2 * D) + 2 * NF * NL + NF * NP;   // ... and [NF][NP] pressure modes
   T* s_misc = s_f + D * FSZ;             // [8]: volume, area
   T(*corner)[3] = reinterpret_cast<T(*)[3]>(s_misc + 8);
+  T* s_psi = s_misc + 8 + 24;            // [Q][NP] pressure modes
   __shared__ int s_faces[6];
   __shared__ int s_nf;
 
@@ -133,6 +143,11 @@ __device__ void elem_cell(const VankaArgs<T>& V, const Tab<T>& tb, int64_t cell,
     T w = det;
     for (int l = 0; l < D; ++l) w *= tb.qw[tq[l]];
     s_jxw[q] = w;
+    for (int m = 0; m < NP; ++m) {
+      T psi = tb.P1[tq[0]][tb.modes[m][0]] * tb.P1[tq[1]][tb.modes[m][1]];
+      if (D == 3) psi *= tb.P1[tq[2]][tb.modes[m][2]];
+      s_psi[q * NP + m] = psi;
+    }
     for (int j = 0; j < NL; ++j) {
       int jm[3]; node_multi<D, N>(j, jm);
       T val = 1, gr[3] = {1, 1, 1};
@@ -195,89 +210,174 @@ __device__ void elem_cell(const VankaArgs<T>& V, const Tab<T>& tb, int64_t cell,
       T y = 0;
       for (int c = 0; c < D; ++c) { f_v[p * D + c] = vv[c]; y += vv[c] * nrm[c]; }
       f_y[p] = y;
+      for (int m = 0; m < NP; ++m) f_dn[NF * NL + p * NP + m] = face_psi<T, D, N>(tb, axis, side, pq, m);
     }
     __syncthreads();
     if (tid == 0) { T a = 0; for (int p = 0; p < NF; ++p) a += f_jxw[p]; s_misc[1 + f] = a; }
     __syncthreads();
   }
-  // velocity block: entry (c, i ; e, j) = row (test c, i), column (trial e, j)
+  // velocity block: entry (c, i ; e, j) = row (test c, i), column (trial e, j).  A thread computes a
+  // tile of TI test nodes x TJ trial nodes for all components: with g_ce = sum_q w v_c phi_j d_e phi_i
+  // the convection part is -(g_ce + delta_ce sum_l g_ll), so per Gauss point and node pair the whole
+  // D x D block costs D^2 + D + 1 multiply-adds on values shared by the tile (3D Q3/P2, 4096 cells:
+  // 9.6 -> 1.2 ms against one matrix entry at a time).
+  constexpr int TI = D == 3 ? 2 : 1, TJ = 4;
+  constexpr int NTI = (NL + TI - 1) / TI, NTJ = (NL + TJ - 1) / TJ;
   T* EA = V.EA + (cell - V.ebase) * (int64_t)MV * MV;
-  for (int ent = tid; ent < MV * MV; ent += nt) {
-    const int row = ent / MV, col = ent % MV;
-    const int c = row / NL, i = row % NL, e = col / NL, j = col % NL;
-    T acc = 0;
-    for (int q = 0; q < Q; ++q) {
-      const T* gi = s_gphi + (q * NL + i) * D;
-      const T* gj = s_gphi + (q * NL + j) * D;
-      const T pj = s_phi[q * NL + j];
-      T t = -s_v[q * D + c] * pj * gi[e];
-      if (c == e) {
-        T lap = 0, adv = 0;
-        for (int l = 0; l < D; ++l) { lap += gi[l] * gj[l]; adv += s_v[q * D + l] * gi[l]; }
-        t += L.nu * lap - pj * adv;
+  T* EM = V.EM + (cell - V.ebase) * (int64_t)NL * NL;
+  for (int tile = tid; tile < NTI * NTJ; tile += nt) {
+    const int i0 = tile / NTJ * TI, j0 = (tile - tile / NTJ * NTJ) * TJ;
+    int in[TI], jn[TJ];                               // nodes past the end repeat the last one and are not stored
+#pragma unroll
+    for (int x = 0; x < TI; ++x) in[x] = i0 + x < NL ? i0 + x : NL - 1;
+#pragma unroll
+    for (int y = 0; y < TJ; ++y) jn[y] = j0 + y < NL ? j0 + y : NL - 1;
+    T g[TI][TJ][D][D], sm_[TI][TJ], mass[TI][TJ];     // sm_: the part common to the diagonal blocks
+#pragma unroll
+    for (int x = 0; x < TI; ++x)
+#pragma unroll
+      for (int y = 0; y < TJ; ++y) {
+        sm_[x][y] = 0;
+        mass[x][y] = 0;
+#pragma unroll
+        for (int c = 0; c < D; ++c)
+#pragma unroll
+          for (int e = 0; e < D; ++e) g[x][y][c][e] = 0;
       }
-      acc += s_jxw[q] * t;
+#pragma unroll 1
+    for (int q = 0; q < Q; ++q) {
+      const T w = s_jxw[q];
+      T wv[D], gi[TI][D], pi[TI];
+#pragma unroll
+      for (int c = 0; c < D; ++c) wv[c] = w * s_v[q * D + c];
+#pragma unroll
+      for (int x = 0; x < TI; ++x) {
+        pi[x] = w * s_phi[q * NL + in[x]];
+#pragma unroll
+        for (int e = 0; e < D; ++e) gi[x][e] = s_gphi[(q * NL + in[x]) * D + e];
+      }
+#pragma unroll
+      for (int y = 0; y < TJ; ++y) {
+        const T pj = s_phi[q * NL + jn[y]];
+        T wg[D], yc[D];
+#pragma unroll
+        for (int e = 0; e < D; ++e) wg[e] = w * s_gphi[(q * NL + jn[y]) * D + e];
+#pragma unroll
+        for (int c = 0; c < D; ++c) yc[c] = wv[c] * pj;
+#pragma unroll
+        for (int x = 0; x < TI; ++x) {
+          mass[x][y] += pi[x] * pj;
+#pragma unroll
+          for (int e = 0; e < D; ++e) {
+            sm_[x][y] += gi[x][e] * wg[e];
+#pragma unroll
+            for (int c = 0; c < D; ++c) g[x][y][c][e] += gi[x][e] * yc[c];
+          }
+        }
+      }
     }
+#pragma unroll
+    for (int x = 0; x < TI; ++x)
+#pragma unroll
+      for (int y = 0; y < TJ; ++y) {
+        T tr = 0;
+#pragma unroll
+        for (int c = 0; c < D; ++c) tr += g[x][y][c][c];
+        sm_[x][y] = L.nu * sm_[x][y] - tr;
+#pragma unroll
+        for (int c = 0; c < D; ++c)
+#pragma unroll
+          for (int e = 0; e < D; ++e) g[x][y][c][e] = -g[x][y][c][e];
+      }
     for (int f = 0; f < nfaces; ++f) {
       const T* F = s_f + f * FSZ;
       const T* f_jxw = F; const T* f_n = F + NF; const T* f_y = f_n + NF * D; const T* f_v = f_y + NF;
       const T* f_phi = f_v + NF * D; const T* f_dn = f_phi + NF * NL;
       const T h = s_misc[0] / s_misc[1 + f] * L.hscale;
+      const T p1 = L.nu * L.gamma1 / h, p2 = L.gamma2 / h;
+#pragma unroll 1
       for (int p = 0; p < NF; ++p) {
-        const T pi = f_phi[p * NL + i], pj = f_phi[p * NL + j];
-        const T y = f_y[p];
-        const T ypos = (T)0.5 * (fabs(y) + y), yneg = (T)0.5 * (fabs(y) - y);
-        const T sgn = (y > 0) ? (T)1 : ((y < 0) ? (T)-1 : (T)0);
-        T t = L.gamma2 / h * f_n[p * D + c] * f_n[p * D + e] * pj * pi;
-        if (c == e) {
-          t += -L.nu * f_dn[p * NL + j] * pi - L.nu * pj * f_dn[p * NL + i] + L.nu * L.gamma1 / h * pj * pi;
-          if (L.bconv) t += (ypos - 2 * yneg) * pj * pi;
+        const T w = f_jxw[p], yn = f_y[p];
+        const T ypos = (T)0.5 * (fabs(yn) + yn), yneg = (T)0.5 * (fabs(yn) - yn);
+        const T sgn = (yn > 0) ? (T)1 : ((yn < 0) ? (T)-1 : (T)0);
+        const T sc = w * (p1 + (L.bconv ? ypos - 2 * yneg : (T)0)), wn = w * L.nu;
+        T K[D][D];
+#pragma unroll
+        for (int c = 0; c < D; ++c)
+#pragma unroll
+          for (int e = 0; e < D; ++e)
+            K[c][e] = w * f_n[p * D + e] *
+                      (p2 * f_n[p * D + c] + (L.bconv ? (T)0.5 * ((T)3 - sgn) * f_v[p * D + c] : (T)0));
+#pragma unroll
+        for (int x = 0; x < TI; ++x) {
+          const T pi = f_phi[p * NL + in[x]], di = f_dn[p * NL + in[x]];
+#pragma unroll
+          for (int y = 0; y < TJ; ++y) {
+            const T pj = f_phi[p * NL + jn[y]], dj = f_dn[p * NL + jn[y]];
+            const T pp = pi * pj;
+            sm_[x][y] += sc * pp - wn * (dj * pi + pj * di);
+#pragma unroll
+            for (int c = 0; c < D; ++c)
+#pragma unroll
+              for (int e = 0; e < D; ++e) g[x][y][c][e] += K[c][e] * pp;
+          }
         }
-        if (L.bconv) t += (T)0.5 * ((T)3 - sgn) * f_n[p * D + e] * pj * f_v[p * D + c] * pi;
-        acc += f_jxw[p] * t;
       }
     }
-    EA[ent] = acc;
+#pragma unroll
+    for (int x = 0; x < TI; ++x)
+#pragma unroll
+      for (int c = 0; c < D; ++c)
+#pragma unroll
+        for (int e = 0; e < D; ++e)
+#pragma unroll
+          for (int y = 0; y < TJ; ++y)
+            if (i0 + x < NL && j0 + y < NL)
+              EA[(int64_t)(c * NL + i0 + x) * MV + e * NL + j0 + y] = g[x][y][c][e] + (c == e ? sm_[x][y] : (T)0);
+#pragma unroll
+    for (int x = 0; x < TI; ++x)
+#pragma unroll
+      for (int y = 0; y < TJ; ++y)
+        if (i0 + x < NL && j0 + y < NL) EM[(i0 + x) * NL + j0 + y] = mass[x][y];
   }
-  // pressure x velocity block B_K[m][(e, j)]
-  const int npc = tb.npc;
-  T* EB = V.EB + (cell - V.ebase) * (int64_t)npc * MV;
-  for (int ent = tid; ent < npc * MV; ent += nt) {
-    const int m = ent / MV, col = ent % MV, e = col / NL, j = col % NL;
-    T acc = 0;
+  // pressure x velocity block B_K[m][(e, j)]: a thread per column, all modes
+  constexpr int NPC = patch_rows<D, N>() - MV;
+  T* EB = V.EB + (cell - V.ebase) * (int64_t)NPC * MV;
+  for (int col = tid; col < MV; col += nt) {
+    const int e = col / NL, j = col - e * NL;
+    T acc[NPC];
+#pragma unroll
+    for (int m = 0; m < NPC; ++m) acc[m] = 0;
+#pragma unroll 1
     for (int q = 0; q < Q; ++q) {
-      int tq[3]; node_multi<D, N>(q, tq);
-      T psi = tb.P1[tq[0]][tb.modes[m][0]] * tb.P1[tq[1]][tb.modes[m][1]];
-      if (D == 3) psi *= tb.P1[tq[2]][tb.modes[m][2]];
-      acc -= s_jxw[q] * psi * s_gphi[(q * NL + j) * D + e];
+      const T w = s_jxw[q] * s_gphi[(q * NL + j) * D + e];
+#pragma unroll
+      for (int m = 0; m < NPC; ++m) acc[m] -= s_psi[q * NPC + m] * w;
     }
     for (int f = 0; f < nfaces; ++f) {
-      const int axis = s_faces[f] / 2, side = s_faces[f] % 2;
       const T* F = s_f + f * FSZ;
       const T* f_jxw = F; const T* f_n = F + NF; const T* f_phi = f_n + NF * D + NF + NF * D;
+      const T* f_psi = f_phi + 2 * NF * NL;
+#pragma unroll 1
       for (int p = 0; p < NF; ++p) {
-        int pq[2] = {p % N, p / N};
-        acc += f_jxw[p] * face_psi<T, D, N>(tb, axis, side, pq, m) * f_n[p * D + e] * f_phi[p * NL + j];
+        const T w = f_jxw[p] * f_n[p * D + e] * f_phi[p * NL + j];
+#pragma unroll
+        for (int m = 0; m < NPC; ++m) acc[m] += f_psi[p * NPC + m] * w;
       }
     }
-    EB[ent] = acc;
-  }
-  T* EM = V.EM + (cell - V.ebase) * (int64_t)NL * NL;
-  for (int ent = tid; ent < NL * NL; ent += nt) {
-    const int i = ent / NL, j = ent % NL;
-    T acc = 0;
-    for (int q = 0; q < Q; ++q) acc += s_jxw[q] * s_phi[q * NL + i] * s_phi[q * NL + j];
-    EM[ent] = acc;
+#pragma unroll
+    for (int m = 0; m < NPC; ++m) EB[m * MV + col] = acc[m];
   }
 }
 
 // Entries of the per-cell tables of elem_cell.
 template <int D, int N>
 __host__ __device__ constexpr size_t elem_table_entries() {
-  return (size_t)Shape<D, N>::Q * Shape<D, N>::Q * D + (size_t)Shape<D, N>::Q * Shape<D, N>::Q + Shape<D, N>::Q +
-         (size_t)Shape<D, N>::Q * D + (size_t)D * Shape<D, N>::Q +
-         (size_t)D * (Shape<D, N>::NF * (2 + 2 * D) + 2 * (size_t)Shape<D, N>::NF * Shape<D, N>::Q) + 8 + 24;
+  constexpr size_t Q = Shape<D, N>::Q, NF = Shape<D, N>::NF, NP = patch_rows<D, N>() - D * Q;
+  return Q * Q * D + Q * Q + Q + Q * D + D * Q + D * (NF * (2 + 2 * D) + 2 * NF * Q + NF * NP) + 8 + 24 + Q * NP;
 }
+// Threads of a block of element matrices: about one node tile each.
+template <int D, int N> __host__ __device__ constexpr int elem_threads() { return D == 2 ? 64 : (N == 3 ? 128 : 256); }
 
 template <typename T, int D, int N>
 __global__ void k_elem(VankaArgs<T> V, Tab<T> tb, int64_t c0, int64_t c1) {
@@ -378,102 +478,6 @@ __device__ bool gauss_jordan(T* S, int m, int ld, int* piv_row, T* colbuf) {
   return true;
 }
 
-// In-place inverse of the complex m x m matrix (Sr + i Si) (row-major, leading dimension m) by
-// Gauss-Jordan elimination with partial pivoting on |a|; same structure as gauss_jordan.
-template <typename T>
-__device__ bool gauss_jordan_c(T* Sr, T* Si, int m, int* piv_row, T* cr, T* ci) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  __shared__ int s_pivc;
-  __shared__ bool s_okc;
-  if (tid == 0) s_okc = true;
-  for (int p = 0; p < m; ++p) {
-    if (tid < 32) {
-      T best = -1; int bi = p;
-      for (int i = p + tid; i < m; i += 32) {
-        const T a = Sr[i * m + p] * Sr[i * m + p] + Si[i * m + p] * Si[i * m + p];
-        if (a > best) { best = a; bi = i; }
-      }
-      for (int off = 16; off > 0; off >>= 1) {
-        T ob = __shfl_down_sync(0xffffffffu, best, off);
-        int oi = __shfl_down_sync(0xffffffffu, bi, off);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (tid == 0) { s_pivc = bi; piv_row[p] = bi; if (!(best > 0)) s_okc = false; }
-    }
-    __syncthreads();
-    if (!s_okc) return false;
-    const int r = s_pivc;
-    if (r != p)
-      for (int j = tid; j < m; j += nt) {
-        T t = Sr[p * m + j]; Sr[p * m + j] = Sr[r * m + j]; Sr[r * m + j] = t;
-        t = Si[p * m + j]; Si[p * m + j] = Si[r * m + j]; Si[r * m + j] = t;
-      }
-    __syncthreads();
-    const T pr = Sr[p * m + p], pi = Si[p * m + p];
-    const T den = (T)1 / (pr * pr + pi * pi);
-    const T qr = pr * den, qi = -pi * den;          // 1 / (pr + i pi)
-    __syncthreads();
-    for (int j = tid; j < m; j += nt) {
-      if (j == p) { Sr[p * m + j] = qr; Si[p * m + j] = qi; }
-      else {
-        const T ar = Sr[p * m + j], ai = Si[p * m + j];
-        Sr[p * m + j] = ar * qr - ai * qi; Si[p * m + j] = ar * qi + ai * qr;
-      }
-    }
-    for (int i = tid; i < m; i += nt) {
-      cr[i] = (i == p) ? (T)0 : Sr[i * m + p];
-      ci[i] = (i == p) ? (T)0 : Si[i * m + p];
-    }
-    __syncthreads();
-    for (int i = tid; i < m; i += nt) if (i != p) { Sr[i * m + p] = 0; Si[i * m + p] = 0; }
-    __syncthreads();
-    if (nt >= m) {
-      const int rs = nt / m;
-      if (tid < rs * m) {
-        const int j = tid % m, chunk = tid / m;
-        const T br = Sr[p * m + j], bim = Si[p * m + j];
-        for (int i0 = chunk; i0 < m; i0 += kGjBatch * rs) {
-          T vr[kGjBatch], vi[kGjBatch];
-#pragma unroll
-          for (int u = 0; u < kGjBatch; ++u) {
-            const int i = i0 + u * rs;
-            vr[u] = i < m ? Sr[i * m + j] : (T)0;
-            vi[u] = i < m ? Si[i * m + j] : (T)0;
-          }
-#pragma unroll
-          for (int u = 0; u < kGjBatch; ++u) {
-            const int i = i0 + u * rs;
-            if (i < m && i != p) {
-              Sr[i * m + j] = vr[u] - (cr[i] * br - ci[i] * bim);
-              Si[i * m + j] = vi[u] - (cr[i] * bim + ci[i] * br);
-            }
-          }
-        }
-      }
-    } else {
-      for (int j = tid; j < m; j += nt) {
-        const T br = Sr[p * m + j], bim = Si[p * m + j];
-        for (int i = 0; i < m; ++i)
-          if (i != p) {
-            Sr[i * m + j] -= cr[i] * br - ci[i] * bim;
-            Si[i * m + j] -= cr[i] * bim + ci[i] * br;
-          }
-      }
-    }
-    __syncthreads();
-  }
-  for (int p = m - 1; p >= 0; --p) {
-    const int r = piv_row[p];
-    if (r != p)
-      for (int i = tid; i < m; i += nt) {
-        T t = Sr[i * m + p]; Sr[i * m + p] = Sr[i * m + r]; Sr[i * m + r] = t;
-        t = Si[i * m + p]; Si[i * m + p] = Si[i * m + r]; Si[i * m + r] = t;
-      }
-    __syncthreads();
-  }
-  return true;
-}
-
 // ---------------------------------------------------------------------------- patch build
 // The cells K' around the cell at cc (offsets o in {-1, 0, 1}^D) that contain both nodes i and j
 // of the cell (multi-indices im, jm within it), visited in the order of the offset code
@@ -508,147 +512,9 @@ __device__ __forceinline__ void for_shared_cells(const int* cc, int n, const int
       }
 }
 
-// Spatial patch ordering: velocity (c, i) -> c*NL + i, then pressure mode m -> MV + m.  The
-// surrogate patch matrix of Eq. vanka0 is, time node by time node,
-//   S~ = [ K^tau (x) M + W (x) A ,  W (x) B^T ;  W (x) B , 0 ],   W = diag(w_a),
-// with the cell's assembled velocity mass M (per component), velocity block A (viscous,
-// convection at v*, Nitsche) and divergence block B.  With W^{-1} K^tau = Q diag(lam) Q^{-1}
-// it is similar to the block diagonal of T_lam = [lam M + A, B^T; B, 0]: one spatial inverse
-// per eigenvalue instead of one inverse of the whole space-time patch (Sec. 4.3).
-template <typename T, int D, int N>
-__device__ bool patch_cell(const VankaArgs<T>& V, const Tab<T>& tb, const TEig<T>& te, int64_t cell, T* Sr, T* Si,
-                           T* Ap, T* Mp, T* cr, T* ci, int* piv) {
-  constexpr int NL = Shape<D, N>::Q;
-  constexpr int MV = D * NL;
-  const int npc = tb.npc, kp1 = tb.k + 1;
-  const int ms = MV + npc, st = inv_stride(ms, V.invh ? 2 : (int)sizeof(T));
-  const LevelArgs<T>& L = V.L;
-  int cc[3] = {0, 0, 0};
-  cell_coords<D>(cell, L.n, cc);
-  const int tid = threadIdx.x, nt = blockDim.x;
-  // assembled velocity and mass blocks: sum over neighbours K' sharing both nodes
-  for (int ent = tid; ent < MV * MV; ent += nt) {
-    const int row = ent / MV, col = ent % MV;
-    const int c = row / NL, i = row % NL, e = col / NL, j = col % NL;
-    int im[3], jm[3];
-    node_multi<D, N>(i, im); node_multi<D, N>(j, jm);
-    T acc = 0;
-    for_shared_cells<D, N>(cc, L.n, im, jm, [&](int64_t nc, int ii, int jj) {
-      acc += V.EA[(nc - V.ebase) * (int64_t)MV * MV + (int64_t)(c * NL + ii) * MV + e * NL + jj];
-    });
-    Ap[ent] = acc;
-  }
-  for (int ent = tid; ent < NL * NL; ent += nt) {
-    const int i = ent / NL, j = ent % NL;
-    int im[3], jm[3];
-    node_multi<D, N>(i, im); node_multi<D, N>(j, jm);
-    T acc = 0;
-    for_shared_cells<D, N>(cc, L.n, im, jm, [&](int64_t nc, int ii, int jj) {
-      acc += V.EM[(nc - V.ebase) * (int64_t)NL * NL + (int64_t)ii * NL + jj];
-    });
-    Mp[ent] = acc;
-  }
-  __syncthreads();
-  const T* EB = V.EB + (cell - V.ebase) * (int64_t)npc * MV;
-  const int64_t cbase = cell * (int64_t)kp1 * ms * st;
-  for (int e = 0; e < te.nblk; ++e) {
-    const bool cplx = te.cplx[e] != 0;
-    const T lr = te.lre[e], li = te.lim[e];
-    for (int ent = tid; ent < ms * ms; ent += nt) {
-      const int row = ent / ms, col = ent % ms;
-      T vr = 0, vi = 0;
-      if (row < MV && col < MV) {
-        vr = Ap[row * MV + col];
-        if (row / NL == col / NL) {
-          const T mm = Mp[(row % NL) * NL + (col % NL)];
-          vr += lr * mm; vi = li * mm;
-        }
-      } else if (row < MV) {
-        vr = EB[(col - MV) * MV + row];
-      } else if (col < MV) {
-        vr = EB[(row - MV) * MV + col];
-      }
-      Sr[ent] = vr;
-      Si[ent] = vi;
-    }
-    __syncthreads();
-    const bool ok = cplx ? gauss_jordan_c<T>(Sr, Si, ms, piv, cr, ci) : gauss_jordan<T>(Sr, ms, ms, piv, cr);
-    if (!ok) { if (tid == 0) *V.status = 1; return false; }
-    const int w = cplx ? 2 : 1;                                  // reals per stored entry
-    const int64_t bbase = cbase + (int64_t)te.off[e] * ms * st;  // in reals
-    if (V.invh) {
-      T mx = 0;
-      for (int ent = tid; ent < ms * ms; ent += nt) mx = fmax(mx, fmax(fabs(Sr[ent]), cplx ? fabs(Si[ent]) : (T)0));
-      mx = block_absmax<T>(mx);
-      // the scale is held in FP32: divide by exactly the value the apply multiplies by
-      const float sc = mx > 0 ? (float)mx : 1.f;
-      const T isc = (T)1 / (T)sc;
-      if (tid == 0) V.scale[cell * te.nblk + e] = sc;
-      __half* inv = V.invh + bbase;
-      for (int ent = tid; ent < ms * st; ent += nt) {
-        const int j = ent / st, i = ent % st;
-        const bool in = i < ms;
-        inv[(int64_t)w * ent] = __float2half_rn(in ? (float)(Sr[i * ms + j] * isc) : 0.f);
-        if (cplx) inv[(int64_t)w * ent + 1] = __float2half_rn(in ? (float)(Si[i * ms + j] * isc) : 0.f);
-      }
-    } else {
-      T* inv = V.inv + bbase;
-      for (int ent = tid; ent < ms * st; ent += nt) {
-        const int j = ent / st, i = ent % st;     // column-major: inv[j][i] = T^{-1}[i][j]
-        const bool in = i < ms;                   // rows ms..st-1 pad the column
-        inv[(int64_t)w * ent] = in ? Sr[i * ms + j] : (T)0;
-        if (cplx) inv[(int64_t)w * ent + 1] = in ? Si[i * ms + j] : (T)0;
-      }
-    }
-    __syncthreads();
-  }
-  return true;
-}
-
-// Patches whose matrices fit shared memory: one block per cell.
-template <typename T, int D, int N>
-__global__ void k_patch(VankaArgs<T> V, Tab<T> tb, TEig<T> te, int64_t c0, int64_t c1) {
-  constexpr int NL = Shape<D, N>::Q;
-  constexpr int MV = D * NL;
-  const int ms = MV + tb.npc;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* Sr = reinterpret_cast<T*>(smem_raw);           // [ms][ms]
-  T* Si = Sr + ms * ms;                             // [ms][ms] imaginary part
-  T* Ap = Si + ms * ms;                             // [MV][MV] assembled velocity block
-  T* Mp = Ap + MV * MV;                             // [NL][NL] assembled scalar mass
-  T* cr = Mp + NL * NL;                             // [ms]
-  T* ci = cr + ms;                                  // [ms]
-  int* piv = reinterpret_cast<int*>(ci + ms);       // [ms]
-  const int64_t cell = c0 + blockIdx.x;
-  if (cell >= c1) return;
-  patch_cell<T, D, N>(V, tb, te, cell, Sr, Si, Ap, Mp, cr, ci, piv);
-}
-
-// Larger patches (3D, r >= 2): the matrices live in a per-block slot of a global workspace
-// (V.work, V.wslot entries per slot; the slots together stay L2-resident); blocks stride over
-// the cells.  Only the pivot bookkeeping is in shared memory.
-template <typename T, int D, int N>
-__global__ void __launch_bounds__(512, 2) k_patch_global(VankaArgs<T> V, Tab<T> tb, TEig<T> te, int64_t c0, int64_t c1) {
-  constexpr int NL = Shape<D, N>::Q;
-  constexpr int MV = D * NL;
-  const int ms = MV + tb.npc;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* cr = reinterpret_cast<T*>(smem_raw);           // [ms]
-  T* ci = cr + ms;                                  // [ms]
-  int* piv = reinterpret_cast<int*>(ci + ms);       // [ms]
-  T* Sr = V.work + (int64_t)blockIdx.x * V.wslot;
-  T* Si = Sr + ms * ms;
-  T* Ap = Si + ms * ms;
-  T* Mp = Ap + MV * MV;
-  for (int64_t cell = c0 + blockIdx.x; cell < c1; cell += gridDim.x) {
-    if (!patch_cell<T, D, N>(V, tb, te, cell, Sr, Si, Ap, Mp, cr, ci, piv)) return;
-    __syncthreads();
-  }
-}
-
 // ---------------------------------------------------------------------------- sweep
 // d[patch] += W~ S~^{-1} res[patch] for the cells of one colour (W~ = omega on velocity,
-// omega_p on pressure DoFs), through the time-diagonalised inverse (k_patch):
+// omega_p on pressure DoFs), through the time-diagonalised inverse (vanka_patch.cuh):
 //   rt_e = sum_a F[e][a] res_a  (per spatial patch DoF),  yhat_e = T_e^{-1} rt_e,
 //   y_a = sum_e Re(G[a][e] yhat_e).
 // One block per cell.  Its inverse ((k+1) m_s x stride reals, contiguous) is staged into shared
@@ -706,13 +572,6 @@ template <> struct InvLd<__half> {
   __device__ static float re(const __half* p) { return __half2float(*p); }
   __device__ static float2 cx(const __half* p) { return __half22float2(*reinterpret_cast<const __half2*>(p)); }
 };
-
-// Rows of the spatial Vanka patch of Q_{N-1} / P_{N-2}^disc: D N^D velocity DoFs and C(r+D, D)
-// pressure modes (r = N - 2), known at compile time so that the row products unroll.
-template <int D, int N>
-__host__ __device__ constexpr int patch_rows() {
-  return D * Shape<D, N>::Q + (D == 2 ? (N - 1) * N / 2 : (N - 1) * N * (N + 1) / 6);
-}
 
 // Dynamic shared memory of k_vanka_apply: [blob | rt (kp1 x mr T) | gb (ms int64) | mbarrier].
 __host__ __device__ inline size_t apply_blob_bytes(int kp1, int ms, size_t si) {

@@ -9,6 +9,7 @@
 #include "mg.hpp"
 #include "op_launch.cuh"
 #include "vanka.cuh"
+#include "vanka_patch.cuh"
 #include "vanka_diag.cuh"
 #include "vanka_exact.cuh"
 #include "vec.cuh"
@@ -20,19 +21,10 @@ namespace stmg {
 
 
 template <int D, int N>
-static size_t elem_smem(size_t es) {
-  constexpr int Q = Shape<D, N>::Q, NL = Q, NF = Shape<D, N>::NF;
-  constexpr int FSZ = NF * (2 + 2 * D) + 2 * NF * NL;
-  return es * (Q * NL * D + Q * NL + Q + Q * D + D * NL + D * FSZ + 8 + 24);
-}
+static constexpr size_t elem_smem(size_t es) { return es * elem_table_entries<D, N>(); }
 
-static size_t patch_smem(const Level& lv, size_t es) {
-  const size_t ms = vanka_spatial_size(lv);
-  size_t nl = 1;
-  for (int l = 0; l < lv.d; ++l) nl *= (lv.r + 2);
-  const size_t mv = lv.d * nl;
-  return es * (2 * ms * ms + mv * mv + nl * nl + 2 * ms) + sizeof(int) * ms + 16;
-}
+// Surrogate patches whose whole elimination runs in registers (k_patch_small).
+static bool patch_small(const Level& lv, size_t es) { return lv.d == 2 && !(es == 8 && lv.r == 3); }
 
 static size_t elem_smem_any(const Level& lv, size_t es) {
   int N = lv.r + 2;
@@ -40,8 +32,12 @@ static size_t elem_smem_any(const Level& lv, size_t es) {
   return N == 3 ? elem_smem<3, 3>(es) : N == 4 ? elem_smem<3, 4>(es) : elem_smem<3, 5>(es);
 }
 
-// The patch matrices of a cell fit shared memory (else k_patch_global, global workspace).
-static bool patch_onchip(const Level& lv, size_t es) { return patch_smem(lv, es) <= 227 * 1024; }
+// The patch matrix of a cell stays on the chip (else a global workspace slot per block).
+static bool patch_onchip(const Level& lv, size_t es) {
+  size_t nl = 1;
+  for (int l = 0; l < lv.d; ++l) nl *= (lv.r + 2);
+  return patch_small(lv, es) || patch_matrix_onchip((int)vanka_spatial_size(lv), (int)nl, es);
+}
 
 // Consumer groups of the warp-specialised persistent apply (k_vanka_apply_ws), which serves 2D
 // patches of more than 32 rows: 5 by default (at most half the stages); the environment variable
@@ -80,15 +76,9 @@ static size_t elem_table_any(const Level& lv) {
 
 // Block slots of the global build workspace and their size in entries.
 constexpr int kWorkSlots = 152 * 2;
-static size_t work_slot(const Level& lv) {
-  const size_t ms = vanka_spatial_size(lv);
-  size_t nl = 1;
-  for (int l = 0; l < lv.d; ++l) nl *= (lv.r + 2);
-  const size_t mv = lv.d * nl;
-  return 2 * ms * ms + mv * mv + nl * nl;
+static size_t work_slot(const Level& lv, size_t es) {
+  return patch_matrix_bytes((int)vanka_spatial_size(lv), es) / es;
 }
-
-
 
 // v* = sum_a phi_a(t*) V^a
 template <typename T>
@@ -108,19 +98,24 @@ static cudaError_t build_dn(const Level& lv, const Problem& pb, const T* U, T* v
   int64_t g = (lv.Nv + 255) / 256; if (g > 152 * 8) g = 152 * 8;
   k_midpoint<T><<<(int)g, 256, 0, s>>>(U, vstar, lv.Nv, lv.k + 1, tb);
   const bool diag = lv.smoother == 1;
-  const bool onchip = diag || patch_onchip(lv, sizeof(T));
-  const bool eon = elem_onchip(lv, sizeof(T));
+  // where the patch matrix and the element tables live follows from (T, D, N) alone
+  constexpr int MS = patch_rows<D, N>(), NLOC = Shape<D, N>::Q;
+  constexpr bool SMALL = D == 2 && !(sizeof(T) == 8 && N == 5);
+  constexpr bool MATRIX_ONCHIP = SMALL || patch_matrix_onchip(MS, NLOC, sizeof(T));
+  constexpr bool eon = elem_smem<D, N>(sizeof(T)) <= 227 * 1024;
+  const bool onchip = diag || MATRIX_ONCHIP;
   if ((!onchip || !eon) && !work) return cudaErrorInvalidValue;
   VankaArgs<T> V{level_args<T>(lv, pb, 0.0), vstar, EA, EB, EM, 0, inv, (__half*)invh, scale, status,
-                 onchip ? nullptr : work, onchip ? 0 : (int64_t)work_slot(lv)};
+                 onchip ? nullptr : work, onchip ? 0 : (int64_t)work_slot(lv, sizeof(T))};
   size_t es = elem_smem<D, N>(sizeof(T));
   cudaError_t e = cudaSuccess;
-  if (eon) {
+  if constexpr (eon) {
     e = allow_smem(k_elem<T, D, N>, es);
     if (e != cudaSuccess) return e;
   }
   size_t ps = 0;
   if (lv.smoother == 2) {
+    if (!eon) return cudaErrorNotSupported;
     const int ms = (int)vanka_spatial_size(lv), mv = ms - lv.npc;
     ps = patch_exact_smem((lv.k + 1) * ms, mv, mv / D, sizeof(T));
     e = allow_smem(k_patch_exact<T, D, N>, ps);
@@ -129,13 +124,11 @@ static cudaError_t build_dn(const Level& lv, const Problem& pb, const T* U, T* v
     ps = patch_diag_smem(lv, sizeof(T));
     e = allow_smem(k_patch_diag<T, D, N>, ps);
     if (e != cudaSuccess) return e;
-  } else if (onchip) {
-    ps = patch_smem(lv, sizeof(T));
-    e = allow_smem(k_patch<T, D, N>, ps);
+  } else if constexpr (!SMALL) {
+    ps = (patch_panel_smem(MS, NLOC, sizeof(T)) + 15) & ~(size_t)15;
+    if (MATRIX_ONCHIP) ps += patch_matrix_bytes(MS, sizeof(T));
+    e = allow_smem(k_patch_blocked<T, D, N, MATRIX_ONCHIP>, ps);
     if (e != cudaSuccess) return e;
-  } else {
-    const size_t ms = vanka_spatial_size(lv);
-    ps = sizeof(T) * 2 * ms + sizeof(int) * ms + 16;
   }
   const TEig<T> te = make_teig<T>(lv.tabs, pb.tau);
   // chunks of whole cell planes (the last coordinate): the element matrices of the chunk and of
@@ -156,14 +149,15 @@ static cudaError_t build_dn(const Level& lv, const Problem& pb, const T* U, T* v
         VankaArgs<T> Va = V;
         Va.vstar = U + (int64_t)a * lv.Nv;
         Va.EA = EA + a * stride;
-        k_elem<T, D, N><<<(unsigned)(e1 - e0), 256, es, s>>>(Va, tb, e0, e1);
+        if constexpr (eon)
+          k_elem<T, D, N><<<(unsigned)(e1 - e0), elem_threads<D, N>(), es, s>>>(Va, tb, e0, e1);
       }
       k_patch_exact<T, D, N><<<(unsigned)(p1 - p0), 256, ps, s>>>(V, tb, stride, p0, p1);
       note_launch(lv.k + 2);
       continue;
     }
-    if (eon) {
-      k_elem<T, D, N><<<(unsigned)(e1 - e0), 256, es, s>>>(V, tb, e0, e1);
+    if constexpr (eon) {
+      k_elem<T, D, N><<<(unsigned)(e1 - e0), elem_threads<D, N>(), es, s>>>(V, tb, e0, e1);
     } else {
       // tables in global memory: one slot per block (the slots precede any patch workspace use,
       // which follows on the same stream)
@@ -174,12 +168,12 @@ static cudaError_t build_dn(const Level& lv, const Problem& pb, const T* U, T* v
     }
     if (diag) {
       k_patch_diag<T, D, N><<<(unsigned)(p1 - p0), 128, ps, s>>>(V, tb, p0, p1);
-    } else if (onchip) {
-      // 3D patches (m_s = 85 for Q2/P1): more threads shorten each elimination step
-      k_patch<T, D, N><<<(unsigned)(p1 - p0), D == 3 ? 512 : 256, ps, s>>>(V, tb, te, p0, p1);
+    } else if constexpr (SMALL) {
+      k_patch_small<T, D, N><<<(unsigned)((p1 - p0 + kSmallCells - 1) / kSmallCells), kSmallCells * small_team<D, N>(), 0, s>>>(
+          V, te, lv.k + 1, p0, p1);
     } else {
-      const int64_t grid = p1 - p0 < kWorkSlots ? p1 - p0 : kWorkSlots;
-      k_patch_global<T, D, N><<<(unsigned)grid, 512, ps, s>>>(V, tb, te, p0, p1);
+      const int64_t grid = MATRIX_ONCHIP || p1 - p0 < kWorkSlots ? p1 - p0 : kWorkSlots;
+      k_patch_blocked<T, D, N, MATRIX_ONCHIP><<<(unsigned)grid, blocked_threads<D, N>(), ps, s>>>(V, te, lv.k + 1, p0, p1);
     }
     note_launch(2);
   }
