@@ -250,12 +250,14 @@ typedef struct {
 stmg_status stmg_set_timing(stmg_handle* h, int on);
 
 /* Failure-handling test hook.  With on != 0, every following Vanka sweep of this handle outside
- * a captured V-cycle arms the shared-memory barrier of its patch staging for 16 bytes more than
- * it copies, so that the kernel's bounded wait runs out: the kernel flags the timeout, waits once
- * more (also bounded) and leaves the correction of that cell unchanged; the call returns
- * STMG_ERR_TIMEOUT.  No copy is left in flight and the GPU is not faulted, so the handle stays
- * usable; on = 0 restores normal operation.  Each sweep launch takes up to a few seconds while
- * the hook is on.  Not part of the method (no counterpart in the paper). */
+ * a captured V-cycle runs a bounded wait into its limit: the sweep with exact patches (smoother = 2)
+ * arms the shared-memory barrier of its patch staging for 16 bytes more than it copies; the other
+ * sweeps, whose kernels wait for nothing, are preceded by one block that waits for bytes never sent.
+ * The kernel flags the timeout (the exact-patch kernel waits once more, also bounded), the correction
+ * is left as it was where the wait failed, and the call returns STMG_ERR_TIMEOUT.  No copy is left in
+ * flight and the GPU is not faulted, so the handle stays usable; on = 0 restores normal operation.
+ * Each sweep launch takes up to a few seconds while the hook is on.  Not part of the method (no
+ * counterpart in the paper). */
 stmg_status stmg_test_wait_timeout(stmg_handle* h, int on);
 
 /* Restrict the per-kernel-class timers of stmg_set_timing to the classes whose bit is set in

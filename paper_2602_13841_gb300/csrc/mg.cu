@@ -167,32 +167,28 @@ cudaError_t MG<T>::sweep(int l, const T* rhs, T* d, int nsweeps, bool zero_start
   const double omega = h->prm.omega;
   for (int it = 0; it < nsweeps; ++it) {
     const T* res = rhs;
-    if (it == 0 && zero_start) {
-      CKE(cudaMemsetAsync(d, 0, (size_t)slots * lv.Nst * sizeof(T), s));
-    } else {
+    const bool first = it == 0 && zero_start;
+    if (!first) {
       // q = rhs - J d
       h->kbegin(KC_APPLYP);
       CKE(launch_level_residual<T>(lv, h->pb, rhs, d, U[l], q[l], s, slots, slots > 1 ? nub : nullptr));
       h->kend(KC_APPLYP);
       res = q[l];
     }
-    // one timer span over the colour launches of the sweep (they run back to back);
+    // one timer span over the launches of the correction;
     // algorithmic bytes: the patch inverses of every cell, residual gather, d read and write
     // per cell: (k+1) m_s^2 stored reals (one spatial inverse per real time eigenvalue, a complex
     // one per conjugate pair), residual gather and d update on the (k+1) m_s patch DoFs
     const double ms = (double)vanka_spatial_size(lv), m = (double)vanka_patch_size(lv);
     const double ib = lv.smoother != 0 ? (double)vanka_inv_entries(lv, (int)sizeof(T)) * sizeof(T)
                       : (lv.k + 1) * ms * ms * (invh[l] ? 2.0 : (double)sizeof(T)) + (invh[l] ? 4.0 * (lv.k + 1) : 0.0);
-    int64_t cells = 0;
+    const int64_t cells = (int64_t)slots * (lv.Np / lv.npc);
     h->kbegin(KC_VANKA_APPLY);
     if (l == 0) h->kbegin(KC_VANKA_APPLY0);
-    for (int c = 0; c < lv.ncolors; ++c) {
-      CKE(vanka_apply<T>(lv, h->pb, inv[l], invh[l], iscale[l], res, d, omega, h->prm.omega_p, c, wstat, s,
-                         h->wait_fault ? 16u : 0u, slots));
-      cells += (int64_t)slots * lv.colors[c].count;
-    }
-    if (l == 0) h->kend(KC_VANKA_APPLY0, (double)cells * (ib + 3.0 * m * sizeof(T)), lv.ncolors);
-    h->kend(KC_VANKA_APPLY, (double)cells * (ib + 3.0 * m * sizeof(T)), lv.ncolors);
+    CKE(vanka_apply<T>(lv, h->pb, inv[l], invh[l], iscale[l], res, d, omega, h->prm.omega_p, wstat, s,
+                       h->wait_fault ? 16u : 0u, slots, first));
+    if (l == 0) h->kend(KC_VANKA_APPLY0, (double)cells * (ib + 3.0 * m * sizeof(T)));
+    h->kend(KC_VANKA_APPLY, (double)cells * (ib + 3.0 * m * sizeof(T)));
   }
   return cudaSuccess;
 }

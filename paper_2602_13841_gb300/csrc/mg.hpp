@@ -80,12 +80,14 @@ cudaError_t vanka_build(const Level& lv, const Problem& pb, const T* U, T* vstar
                         T* inv, void* invh, float* scale, int* status, T* work, cudaStream_t s);
 size_t vanka_work_entries(const Level& lv, size_t esize);  // global build workspace (0: on-chip patches)
 size_t vanka_elem_cells(const Level& lv);   // cells per chunk of the element-matrix scratch
-// inv: patch inverses of precision T, or (invh non-null) FP16 inverses scaled by scale[cell].
+// One Vanka correction d <- d + W sum_K R_K^T S~_K^{-1} R_K res over all cells.  inv: patch inverses of
+// precision T, or (invh non-null) FP16 inverses scaled by scale[cell].  first: d is zero on entry (not read).
 template <typename T>
 cudaError_t vanka_apply(const Level& lv, const Problem& pb, const T* inv, const void* invh, const float* scale,
-                        const T* res, T* d, double omega, double omega_p, int color, int* wstat, cudaStream_t s,
+                        const T* res, T* d, double omega, double omega_p, int* wstat, cudaStream_t s,
                         unsigned extra_tx = 0,    // extra_tx: failure-test hook (see stmg_test_wait_timeout)
-                        int slots = 1);           // independent slots: inverses, res and d at slot strides
+                        int slots = 1,            // independent slots: inverses, res and d at slot strides
+                        bool first = false);
 size_t vanka_spatial_size(const Level& lv);          // m_s = d (r+2)^d + npc
 size_t vanka_patch_size(const Level& lv);            // m_st = (k+1) m_s
 size_t vanka_inv_entries(const Level& lv, int es);   // stored reals of one cell's patch inverse ((k+1) m_s x stride), es-byte entries

@@ -44,20 +44,16 @@ static cudaError_t sweep_noalloc(Handle* h, MG<T>& mg, int l, const T* rhs, T* d
   const Level& lv = h->levels[l];
   for (int it = 0; it < nsweeps; ++it) {
     const T* res = rhs;
-    if (it == 0 && zero_start) {
-      cudaError_t e = cudaMemsetAsync(d, 0, lv.Nst * sizeof(T), s);
-      if (e != cudaSuccess) return e;
-    } else {
+    const bool first = it == 0 && zero_start;
+    if (!first) {
       // q = rhs - J d, by the same launches as the regular sweep
       cudaError_t e = launch_level_residual<T>(lv, h->pb, rhs, d, mg.U[l], q, s);
       if (e != cudaSuccess) return e;
       res = q;
     }
-    for (int c = 0; c < lv.ncolors; ++c) {
-      cudaError_t e = vanka_apply<T>(lv, h->pb, mg.inv[l], mg.invh[l], mg.iscale[l], res, d, h->prm.omega,
-                                     h->prm.omega_p, c, mg.wstat, s, h->wait_fault ? 16u : 0u);
-      if (e != cudaSuccess) return e;
-    }
+    cudaError_t e = vanka_apply<T>(lv, h->pb, mg.inv[l], mg.invh[l], mg.iscale[l], res, d, h->prm.omega, h->prm.omega_p,
+                                   mg.wstat, s, h->wait_fault ? 16u : 0u, 1, first);
+    if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }

@@ -40,6 +40,40 @@ inline int cells_per_block(int threads_per_cell, int max_threads, int64_t cells)
   return spread < best ? (int)spread : best;
 }
 
+// The level's cell buffer for `batch` columns: columns per pass and cell planes per launch -- whole
+// columns while they fit, else one column at a time in chunks of planes.
+template <typename T, int D, int N>
+static bool plan_cellbuf(const Level& lv, int batch, CellBuf<T>& cb, int64_t& cols, int& step) {
+  const int kp1 = lv.k + 1;
+  const int64_t cplane = D == 2 ? lv.n : (int64_t)lv.n * lv.n;
+  cb.s = (T*)lv.cellbuf;
+  cb.plane = cplane * Shape<D, N>::Q;
+  const int64_t cap = (int64_t)(lv.cellbuf_bytes / sizeof(T)), per = (int64_t)kp1 * D * cb.plane;
+  const bool whole = per * lv.n <= cap;
+  cb.P = whole ? lv.n : (int)(cap / per);
+  if (!cb.s || (!whole && cb.P < 2)) return false;
+  cb.comp = cb.plane * cb.P;
+  cb.col = cb.comp * kp1 * D;
+  cols = whole ? cap / cb.col : 1;
+  if (cols > batch) cols = batch;
+  if (cols > 32768) cols = 32768;
+  step = whole ? lv.n : cb.P - 1;
+  return true;
+}
+
+// Node sums of the cell planes z0 .. z1 - 1 (see k_node_sum).
+template <typename T, int D, int N>
+static void launch_node_sum(const Level& lv, const CellBuf<T>& cb, const T* src, T* y, T alpha, int64_t ys, int z0,
+                            int z1, int columns, const int* skip, cudaStream_t s) {
+  const int g0 = z0 * (N - 1), g1 = z1 == lv.n ? lv.N1 : z1 * (N - 1);
+  const int64_t nodes = (int64_t)(g1 - g0) * (D == 2 ? (int64_t)lv.N1 : (int64_t)lv.N1 * lv.N1);
+  const int64_t blocks = (nodes + 127) / 128;
+  auto kern = lv.k == 0 ? k_node_sum<T, D, N, 1> : lv.k == 1 ? k_node_sum<T, D, N, 2> : k_node_sum<T, D, N, 3>;
+  kern<<<dim3((unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), columns), 128, 0, s>>>(
+      cb, src, y, alpha, lv.n, lv.N1, lv.nnodes, lv.Nv, ys, g0, nodes, skip);
+  note_launch();
+}
+
 // One operator call in two launches per chunk (cells, node sums): whole columns while they fit the
 // level's cell buffer, else one column at a time in chunks of cell planes.
 template <typename T, int D, int N, int MODE>
@@ -58,18 +92,9 @@ static cudaError_t launch_dn(const Level& lv, const Problem& pb, double t0, cons
   }
   const int64_t cplane = D == 2 ? lv.n : (int64_t)lv.n * lv.n;   // cells per plane of the last axis
   CellBuf<T> cb{};
-  cb.s = (T*)lv.cellbuf;
-  cb.plane = cplane * Shape<D, N>::Q;
-  const int64_t cap = (int64_t)(lv.cellbuf_bytes / sizeof(T)), per = (int64_t)kp1 * D * cb.plane;
-  const bool whole = per * lv.n <= cap;
-  cb.P = whole ? lv.n : (int)(cap / per);
-  if (!cb.s || cb.P < 2) { if (!(whole && cb.s)) return cudaErrorInvalidValue; }
-  cb.comp = cb.plane * cb.P;
-  cb.col = cb.comp * kp1 * D;
-  int64_t cols = whole ? cap / cb.col : 1;
-  if (cols > batch) cols = batch;
-  if (cols > 32768) cols = 32768;
-  const int step = whole ? lv.n : cb.P - 1;
+  int64_t cols;
+  int step;
+  if (!plan_cellbuf<T, D, N>(lv, batch, cb, cols, step)) return cudaErrorInvalidValue;
   auto kern = [] {
     if constexpr (D == 2) return k_cells2d<T, N, MODE, BT, MINB>; else return k_cells3d<T, N, MODE, BT, MINB>;
   }();
@@ -89,12 +114,8 @@ static cudaError_t launch_dn(const Level& lv, const Problem& pb, double t0, cons
       }
       const int threads = (cpb * kp1 * TPG + 31) / 32 * 32;
       kern<<<dim3((unsigned)((c1 - c0 + cpb - 1) / cpb), nb), threads, smem, stream>>>(A, tb, cb, c0, c1, cpb, rb);
-      const int g0 = z0 * (N - 1), g1 = z1 == lv.n ? lv.N1 : z1 * (N - 1);
-      const int64_t nodes = (int64_t)(g1 - g0) * (D == 2 ? (int64_t)lv.N1 : (int64_t)lv.N1 * lv.N1);
-      const int64_t blocks = (nodes + 127) / 128;
-      k_node_sum<T, D, N><<<dim3((unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), nb), 128, 0, stream>>>(
-          cb, rb, A.y, lv.n, lv.N1, lv.nnodes, lv.Nv, kp1, ys, g0, nodes);
-      note_launch(2);
+      note_launch();
+      launch_node_sum<T, D, N>(lv, cb, rb, A.y, rhs ? (T)-1 : (T)1, ys, z0, z1, nb, nullptr, stream);
     }
   }
   return cudaGetLastError();

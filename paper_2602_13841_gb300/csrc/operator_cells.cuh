@@ -1277,14 +1277,15 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
 }
 
 // ---------------------------------------------------------------------------- node sums
-// y (velocity part, node planes g0 .. g1-1 of the last axis) = the sum of the cells' contributions
-// at each node, or rhs minus it.  One thread per node, all components and time nodes; the cells
-// of a node in ascending order.
-template <typename T, int D, int N>
-__global__ void k_node_sum(CellBuf<T> cb, const T* __restrict__ rhs, T* __restrict__ y, int n, int N1, int64_t nnodes,
-                           int64_t Nv, int kp1, int64_t ys, int g0, int64_t count) {
+// y (velocity part, node planes g0 .. g1-1 of the last axis) = src + alpha * the sum of the cells'
+// contributions at each node (src null: zero; src may be y).  One thread per node, all components and
+// time nodes; the cells of a node in ascending order.  skip: a set flag leaves y as it is.
+template <typename T, int D, int N, int KP1>
+__global__ void k_node_sum(CellBuf<T> cb, const T* src, T* y, T alpha, int n, int N1, int64_t nnodes, int64_t Nv,
+                           int64_t ys, int g0, int64_t count, const int* skip) {
+  if (skip && *skip) return;
   y += blockIdx.y * ys;
-  if (rhs) rhs += blockIdx.y * ys;
+  if (src) src += blockIdx.y * ys;
   const T* s = cb.s + blockIdx.y * cb.col;
   const int64_t row = (int64_t)n * N;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < count; t += (int64_t)gridDim.x * blockDim.x) {
@@ -1312,22 +1313,25 @@ __global__ void k_node_sum(CellBuf<T> cb, const T* __restrict__ rhs, T* __restri
       o1[l] = two[l] ? at(c, 0) : 0;
     }
     const int64_t node = gm[0] + (int64_t)N1 * (gm[1] + (int64_t)N1 * gm[2]);
-#pragma unroll 3
-    for (int ac = 0; ac < kp1 * D; ++ac) {
+    T old[KP1 * D], v[KP1 * D];
+#pragma unroll
+    for (int ac = 0; ac < KP1 * D; ++ac) {
+      old[ac] = src ? src[(int64_t)(ac / D) * Nv + (int64_t)(ac % D) * nnodes + node] : (T)0;
       const T* sc = s + (int64_t)ac * cb.comp;
-      T acc = 0;
+      v[ac] = 0;
 #pragma unroll
       for (int k2 = 0; k2 < (D == 3 ? 2 : 1); ++k2)
 #pragma unroll
         for (int k1 = 0; k1 < 2; ++k1) {
-          if ((k2 && !two[2]) || (k1 && !two[1])) continue;
+          const bool on = !(k2 && !two[2]) && !(k1 && !two[1]);
           const T* q = sc + (k1 ? o1[1] : o0[1]) + (k2 ? o1[2] : o0[2]);
-          acc += q[o0[0]];
-          if (two[0]) acc += q[o1[0]];
+          v[ac] += on ? q[o0[0]] : (T)0;
+          v[ac] += on && two[0] ? q[o1[0]] : (T)0;
         }
-      const int64_t gi = (int64_t)(ac / D) * Nv + (int64_t)(ac % D) * nnodes + node;
-      y[gi] = rhs ? rhs[gi] - acc : acc;
     }
+#pragma unroll
+    for (int ac = 0; ac < KP1 * D; ++ac)
+      y[(int64_t)(ac / D) * Nv + (int64_t)(ac % D) * nnodes + node] = old[ac] + alpha * v[ac];
   }
 }
 

@@ -10,8 +10,8 @@ namespace stmg {
   extern template cudaError_t vanka_build_dim<T, D>(const Level&, const Problem&, const T*, T*, T*, T*, T*, T*,  \
                                                     void*, float*, int*, T*, cudaStream_t);                       \
   extern template cudaError_t vanka_apply_dim<T, D>(const Level&, const Problem&, const T*, const void*,         \
-                                                    const float*, const T*, T*, double, double, int, int*,       \
-                                                    cudaStream_t, unsigned, int);
+                                                    const float*, const T*, T*, double, double, int*,            \
+                                                    cudaStream_t, unsigned, int, bool);
 STMG_EXTERN(float, 2)
 STMG_EXTERN(double, 2)
 STMG_EXTERN(float, 3)
@@ -86,10 +86,10 @@ cudaError_t vanka_build(const Level& lv, const Problem& pb, const T* U, T* vstar
 
 template <typename T>
 cudaError_t vanka_apply(const Level& lv, const Problem& pb, const T* inv, const void* invh, const float* scale,
-                        const T* res, T* d, double omega, double omega_p, int color, int* wstat, cudaStream_t s,
-                        unsigned extra_tx, int slots) {
-  return lv.d == 2 ? vanka_apply_dim<T, 2>(lv, pb, inv, invh, scale, res, d, omega, omega_p, color, wstat, s, extra_tx, slots)
-                   : vanka_apply_dim<T, 3>(lv, pb, inv, invh, scale, res, d, omega, omega_p, color, wstat, s, extra_tx, slots);
+                        const T* res, T* d, double omega, double omega_p, int* wstat, cudaStream_t s,
+                        unsigned extra_tx, int slots, bool first) {
+  return lv.d == 2 ? vanka_apply_dim<T, 2>(lv, pb, inv, invh, scale, res, d, omega, omega_p, wstat, s, extra_tx, slots, first)
+                   : vanka_apply_dim<T, 3>(lv, pb, inv, invh, scale, res, d, omega, omega_p, wstat, s, extra_tx, slots, first);
 }
 
 template cudaError_t vanka_build<float>(const Level&, const Problem&, const float*, float*, float*, float*, float*,
@@ -97,8 +97,8 @@ template cudaError_t vanka_build<float>(const Level&, const Problem&, const floa
 template cudaError_t vanka_build<double>(const Level&, const Problem&, const double*, double*, double*, double*,
                                          double*, double*, void*, float*, int*, double*, cudaStream_t);
 template cudaError_t vanka_apply<float>(const Level&, const Problem&, const float*, const void*, const float*,
-                                        const float*, float*, double, double, int, int*, cudaStream_t, unsigned, int);
+                                        const float*, float*, double, double, int*, cudaStream_t, unsigned, int, bool);
 template cudaError_t vanka_apply<double>(const Level&, const Problem&, const double*, const void*, const float*,
-                                         const double*, double*, double, double, int, int*, cudaStream_t, unsigned, int);
+                                         const double*, double*, double, double, int*, cudaStream_t, unsigned, int, bool);
 
 }  // namespace stmg

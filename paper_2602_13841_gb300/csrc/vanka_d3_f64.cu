@@ -7,6 +7,6 @@ namespace stmg {
 template cudaError_t vanka_build_dim<double, 3>(const Level&, const Problem&, const double*, double*, double*, double*, double*, double*,
                                               void*, float*, int*, double*, cudaStream_t);
 template cudaError_t vanka_apply_dim<double, 3>(const Level&, const Problem&, const double*, const void*, const float*,
-                                              const double*, double*, double, double, int, int*, cudaStream_t, unsigned, int);
+                                              const double*, double*, double, double, int*, cudaStream_t, unsigned, int, bool);
 
 }  // namespace stmg

@@ -1,15 +1,14 @@
 // Vanka launch templates shared by the per-dimension translation units (vanka_d2_*.cu,
 // vanka_d3_*.cu) and the dispatch in vanka.cu: shared-memory budgets, the build of one level and
-// the colour launches of one sweep, per element type T, dimension D and N = r + 2.
+// the launches of one sweep, per element type T, dimension D and N = r + 2.
 #pragma once
-#include <cstdlib>
-#include <cstring>
 #include <type_traits>
 
 #include "mg.hpp"
 #include "op_launch.cuh"
 #include "vanka.cuh"
 #include "vanka_patch.cuh"
+#include "vanka_stream.cuh"
 #include "vanka_diag.cuh"
 #include "vanka_exact.cuh"
 #include "vec.cuh"
@@ -37,25 +36,6 @@ static bool patch_onchip(const Level& lv, size_t es) {
   size_t nl = 1;
   for (int l = 0; l < lv.d; ++l) nl *= (lv.r + 2);
   return patch_small(lv, es) || patch_matrix_onchip((int)vanka_spatial_size(lv), (int)nl, es);
-}
-
-// Consumer groups of the warp-specialised persistent apply (k_vanka_apply_ws), which serves 2D
-// patches of more than 32 rows: 5 by default (at most half the stages); the environment variable
-// STMG_VANKA_WS overrides it (0: one-shot k_vanka_apply blocks, kept for comparisons; read once).
-inline int vanka_ws_groups() {
-  static const int c = [] {
-    const char* v = std::getenv("STMG_VANKA_WS");
-    if (!v) return 5;
-    const int x = std::atoi(v);
-    return x < 0 ? 0 : (x > 8 ? 8 : x);
-  }();
-  return c;
-}
-inline bool vanka_ws_enabled() { return vanka_ws_groups() > 0; }
-
-// The stored inverse blob of a cell fits shared memory (else k_vanka_apply_global).
-static bool apply_onchip(const Level& lv, size_t es_store, size_t es) {
-  return apply_slot_bytes(lv.k + 1, (int)vanka_spatial_size(lv), es_store, es) <= 227 * 1024;
 }
 
 // Shared memory of k_patch_diag: inverse temporal blocks, Schur complement, pivots, column.
@@ -181,107 +161,89 @@ static cudaError_t build_dn(const Level& lv, const Problem& pb, const T* U, T* v
   return cudaGetLastError();
 }
 
+// d <- d + omega W y over all cells of a level by the streamed inverses (first: d = 0 on entry).
 template <typename T, typename SI, int D, int N>
-static cudaError_t apply_cells(const Level& lv, const Problem& pb, const SI* inv, const float* scale, const T* res,
-                               T* d, double omega, double omega_p, const ColorInfo& ci, int* wstat,
-                               unsigned extra_tx, cudaStream_t s, int slots, SlotStrides zs) {
-  // one block per cell, threads = spatial patch rows rounded up to whole warps
-  const int ms = (int)vanka_spatial_size(lv), kp1 = lv.k + 1;
-  if (ms != patch_rows<D, N>()) return cudaErrorInvalidValue;
-  const int threads = ((ms + 31) / 32) * 32;
-  if (!apply_onchip(lv, sizeof(SI), sizeof(T))) {
-    const int mr = (ms + 1) & ~1;
-    const size_t gsm = (((size_t)kp1 * mr * sizeof(T) + 7) & ~(size_t)7) + (size_t)ms * 8;
-    k_vanka_apply_global<T, SI, D, N><<<dim3((unsigned)ci.count, slots), threads, gsm, s>>>(
-        level_args<T>(lv, pb, 0.0), inv, scale, res, d, (T)omega, (T)omega_p, kp1, lv.npc,
-        make_teig<T>(lv.tabs, pb.tau), ci, zs);
-    return cudaSuccess;
+static cudaError_t apply_stream(const Level& lv, const Problem& pb, const SI* inv, const float* scale, const T* res,
+                                T* d, double omega, double omega_p, int* wstat, unsigned extra_tx, cudaStream_t s,
+                                int slots, SlotStrides zs, bool first) {
+  using Sh = StreamShape<T, SI, D, N>;
+  if ((int)vanka_spatial_size(lv) != Sh::MS) return cudaErrorInvalidValue;
+  const int kp1 = lv.k + 1;
+  CellBuf<T> cb{};
+  int64_t cols;
+  int step;
+  if (!plan_cellbuf<T, D, N>(lv, slots, cb, cols, step)) return cudaErrorInvalidValue;
+  const int64_t cplane = D == 2 ? lv.n : (int64_t)lv.n * lv.n;
+  // inverses beyond half of the 129 MB L2 are streamed past it
+  const int64_t bytes = cplane * lv.n * (int64_t)kp1 * Sh::MS * Sh::ST * (int64_t)sizeof(SI);
+  const int stream = bytes * slots > (int64_t)64 << 20;
+  const LevelArgs<T> L = level_args<T>(lv, pb, 0.0);
+  const TEig<T> te = make_teig<T>(lv.tabs, pb.tau);
+  // the kernel's blocks: one real (k = 0), one complex pair (k = 1), one of each (k = 2)
+  const int pairs = te.cplx[0] + (te.nblk > 1 ? te.cplx[1] : 0);
+  if (te.nblk != (kp1 + 1) / 2 || pairs != kp1 / 2) return cudaErrorNotSupported;
+  auto kern = kp1 == 1 ? k_vanka_stream<T, SI, D, N, 1> : kp1 == 2 ? k_vanka_stream<T, SI, D, N, 2> : k_vanka_stream<T, SI, D, N, 3>;
+  if (extra_tx) {
+    k_wait_hook<<<1, 1, 0, s>>>(wstat, extra_tx);
+    note_launch();
   }
-  // 2D patches of more than one warp's rows: the warp-specialised persistent kernel, one block
-  // per SM, as many stages as fit 200 KB of shared memory
-  if constexpr (D == 2) {
-    if (threads > 32 && vanka_ws_enabled()) {
-      const size_t blob = apply_blob_bytes(kp1, ms, sizeof(SI));
-      const size_t rtb = ws_rt_bytes(kp1, ms, sizeof(T));
-      const int cw = vanka_ws_groups();
-      int S = (int)((200 * 1024 - cw * rtb - 16) / (blob + 16));
-      if (S > 16) S = 16;
-      int C = S >= 2 * cw ? cw : S / 2;
-      // the block's registers must fit the SM's 64 K
-      cudaFuncAttributes fa{};
-      cudaError_t e = cudaFuncGetAttributes(&fa, k_vanka_apply_ws<T, SI, D, N>);
-      if (e != cudaSuccess) return e;
-      const int regs = (fa.numRegs + 7) & ~7;        // allocation granularity
-      while (C > 1 && ((32 + C * threads) * regs > 65536 || 32 + C * threads > fa.maxThreadsPerBlock)) --C;
-      if (C >= 1 && (32 + C * threads) * regs <= 65536 && 32 + C * threads <= fa.maxThreadsPerBlock) {
-        const size_t wsm = ws_smem_bytes(kp1, ms, sizeof(SI), sizeof(T), S, C);
-        e = allow_smem(k_vanka_apply_ws<T, SI, D, N>, wsm);
-        if (e != cudaSuccess) return e;
-        int dev = 0, sms = 0;
-        e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        const unsigned grid = (unsigned)(ci.count < sms ? ci.count : sms);
-        k_vanka_apply_ws<T, SI, D, N><<<dim3(grid, slots), 32 + C * threads, wsm, s>>>(
-            level_args<T>(lv, pb, 0.0), inv, scale, res, d, (T)omega, (T)omega_p, kp1, lv.npc,
-            make_teig<T>(lv.tabs, pb.tau), ci, wstat, extra_tx, zs, S, C, threads);
-        return cudaSuccess;
-      }
+  for (int b0 = 0; b0 < slots; b0 += (int)cols) {
+    const int nb = slots - b0 < (int)cols ? slots - b0 : (int)cols;
+    const T* rb = res + b0 * zs.vec;
+    T* db = d + b0 * zs.vec;
+    for (int z0 = 0; z0 < lv.n; z0 += step) {
+      const int z1 = z0 + step < lv.n ? z0 + step : lv.n;
+      kern<<<dim3((unsigned)((z1 - z0) * cplane), nb), Sh::THREADS, 0, s>>>(
+          L, inv + b0 * zs.inv, scale ? scale + b0 * zs.scale : nullptr, rb, db, (T)omega_p, te, cb, z0 * cplane, zs, first,
+          stream);
+      note_launch();
+      launch_node_sum<T, D, N>(lv, cb, first ? nullptr : db, db, (T)omega, zs.vec, z0, z1, nb, wstat, s);
     }
   }
-  // cells per block: 4 for one-warp patches (32 resident blocks per SM), else 1
-  const size_t slot = apply_slot_bytes(kp1, ms, sizeof(SI), sizeof(T));
-  int cpb = threads <= 32 ? 4 : 1;
-  while (cpb > 1 && (size_t)cpb * slot > 100 * 1024) cpb /= 2;
-  const size_t smem = (size_t)cpb * slot;
-  cudaError_t e = allow_smem(k_vanka_apply<T, SI, D, N>, smem);
-  if (e != cudaSuccess) return e;
-  const unsigned blocks = (unsigned)((ci.count + cpb - 1) / cpb);
-  k_vanka_apply<T, SI, D, N><<<dim3(blocks, slots), threads * cpb, smem, s>>>(
-      level_args<T>(lv, pb, 0.0), inv, scale, res, d, (T)omega, (T)omega_p, kp1, lv.npc,
-      make_teig<T>(lv.tabs, pb.tau), ci, wstat, extra_tx, zs);
-  return cudaSuccess;
+  return cudaGetLastError();
 }
 
 template <typename T, int D, int N>
 static cudaError_t apply_dn(const Level& lv, const Problem& pb, const T* inv, const void* invh, const float* scale,
-                            const T* res, T* d, double omega, double omega_p, int color, int* wstat,
-                            unsigned extra_tx, cudaStream_t s, int slots) {
-  const ColorInfo& ci = lv.colors[color];
-  if (ci.count == 0) return cudaSuccess;
+                            const T* res, T* d, double omega, double omega_p, int* wstat, unsigned extra_tx,
+                            cudaStream_t s, int slots, bool first) {
   const int64_t cells = lv.Np / lv.npc;
   const SlotStrides zs{cells * (int64_t)vanka_inv_entries(lv, invh ? 2 : (int)sizeof(T)), cells * (lv.k + 1),
                        lv.Nst};
-  if (lv.smoother == 2) {
-    const int ms = (int)vanka_spatial_size(lv), mst = (lv.k + 1) * ms;
-    const size_t smem = apply_exact_smem(mst, ms, sizeof(T));
-    cudaError_t e = allow_smem(k_vanka_apply_exact<T, D, N>, smem);
+  if (lv.smoother == 0)
+    return invh ? apply_stream<T, __half, D, N>(lv, pb, (const __half*)invh, scale, res, d, omega, omega_p, wstat,
+                                                extra_tx, s, slots, zs, first)
+                : apply_stream<T, T, D, N>(lv, pb, inv, nullptr, res, d, omega, omega_p, wstat, extra_tx, s, slots, zs,
+                                           first);
+  if (first) {
+    cudaError_t e = cudaMemsetAsync(d, 0, (size_t)slots * lv.Nst * sizeof(T), s);
     if (e != cudaSuccess) return e;
-    k_vanka_apply_exact<T, D, N><<<dim3((unsigned)ci.count, slots), ((mst + 31) / 32) * 32, smem, s>>>(
-        level_args<T>(lv, pb, 0.0), inv, res, d, (T)omega, (T)omega_p, lv.k + 1, lv.npc, ci, wstat, extra_tx, zs);
-    note_launch();
-    return cudaGetLastError();
   }
-  if (lv.smoother == 1) {
-    // diagonal space-time Vanka: one warp per cell, up to four cells per block
-    constexpr int NL = Shape<D, N>::Q;
-    const size_t slot = diag_slot_bytes(D * NL, lv.npc, lv.k + 1, sizeof(T));
-    int cpb = 4;
-    while (cpb > 1 && (size_t)cpb * slot > 200 * 1024) --cpb;
-    const size_t smem = (size_t)cpb * slot;
-    cudaError_t e = allow_smem(k_vanka_apply_diag<T, D, N>, smem);
-    if (e != cudaSuccess) return e;
-    k_vanka_apply_diag<T, D, N><<<dim3((unsigned)((ci.count + cpb - 1) / cpb), slots), 32 * cpb, smem, s>>>(
-        level_args<T>(lv, pb, 0.0), inv, res, d, (T)omega, (T)omega_p, make_tab<T>(lv.tabs, pb.tau), ci, cpb, zs);
+  // the other smoothers scatter in place, colour by colour
+  for (int c = 0; c < lv.ncolors; ++c) {
+    const ColorInfo& ci = lv.colors[c];
+    if (ci.count == 0) continue;
+    if (lv.smoother == 2) {
+      const int ms = (int)vanka_spatial_size(lv), mst = (lv.k + 1) * ms;
+      const size_t smem = apply_exact_smem(mst, ms, sizeof(T));
+      cudaError_t e = allow_smem(k_vanka_apply_exact<T, D, N>, smem);
+      if (e != cudaSuccess) return e;
+      k_vanka_apply_exact<T, D, N><<<dim3((unsigned)ci.count, slots), ((mst + 31) / 32) * 32, smem, s>>>(
+          level_args<T>(lv, pb, 0.0), inv, res, d, (T)omega, (T)omega_p, lv.k + 1, lv.npc, ci, wstat, extra_tx, zs);
+    } else {
+      // diagonal space-time Vanka: one warp per cell, up to four cells per block
+      constexpr int NL = Shape<D, N>::Q;
+      const size_t slot = diag_slot_bytes(D * NL, lv.npc, lv.k + 1, sizeof(T));
+      int cpb = 4;
+      while (cpb > 1 && (size_t)cpb * slot > 200 * 1024) --cpb;
+      const size_t smem = (size_t)cpb * slot;
+      cudaError_t e = allow_smem(k_vanka_apply_diag<T, D, N>, smem);
+      if (e != cudaSuccess) return e;
+      k_vanka_apply_diag<T, D, N><<<dim3((unsigned)((ci.count + cpb - 1) / cpb), slots), 32 * cpb, smem, s>>>(
+          level_args<T>(lv, pb, 0.0), inv, res, d, (T)omega, (T)omega_p, make_tab<T>(lv.tabs, pb.tau), ci, cpb, zs);
+    }
     note_launch();
-    return cudaGetLastError();
   }
-  cudaError_t e = invh ? apply_cells<T, __half, D, N>(lv, pb, (const __half*)invh, scale, res, d, omega, omega_p, ci,
-                                                      wstat, extra_tx, s, slots, zs)
-                       : apply_cells<T, T, D, N>(lv, pb, inv, nullptr, res, d, omega, omega_p, ci, wstat, extra_tx,
-                                                 s, slots, zs);
-  if (e != cudaSuccess) return e;
-  note_launch();
   return cudaGetLastError();
 }
 
@@ -299,12 +261,12 @@ cudaError_t vanka_build_dim(const Level& lv, const Problem& pb, const T* U, T* v
 
 template <typename T, int D>
 cudaError_t vanka_apply_dim(const Level& lv, const Problem& pb, const T* inv, const void* invh, const float* scale,
-                            const T* res, T* d, double omega, double omega_p, int color, int* wstat, cudaStream_t s,
-                            unsigned extra_tx, int slots) {
+                            const T* res, T* d, double omega, double omega_p, int* wstat, cudaStream_t s,
+                            unsigned extra_tx, int slots, bool first) {
   const int N = lv.r + 2;
-  if (N == 3) return apply_dn<T, D, 3>(lv, pb, inv, invh, scale, res, d, omega, omega_p, color, wstat, extra_tx, s, slots);
-  if (N == 4) return apply_dn<T, D, 4>(lv, pb, inv, invh, scale, res, d, omega, omega_p, color, wstat, extra_tx, s, slots);
-  if (N == 5) return apply_dn<T, D, 5>(lv, pb, inv, invh, scale, res, d, omega, omega_p, color, wstat, extra_tx, s, slots);
+  if (N == 3) return apply_dn<T, D, 3>(lv, pb, inv, invh, scale, res, d, omega, omega_p, wstat, extra_tx, s, slots, first);
+  if (N == 4) return apply_dn<T, D, 4>(lv, pb, inv, invh, scale, res, d, omega, omega_p, wstat, extra_tx, s, slots, first);
+  if (N == 5) return apply_dn<T, D, 5>(lv, pb, inv, invh, scale, res, d, omega, omega_p, wstat, extra_tx, s, slots, first);
   return cudaErrorNotSupported;
 }
 
