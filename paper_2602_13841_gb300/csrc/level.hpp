@@ -22,8 +22,7 @@ struct Level {
   double hscale = 0;                  // Nitsche length factor (see LevelArgs)
   int64_t chunk_cells = 262144;       // cells per chunk of the smoother build's element scratch
   int smoother = 0;                   // 0: surrogate patches (Sec. 4.3); 1: diagonal space-time Vanka
-  double* geo64 = nullptr;            // 2D: geometry table of the Jacobian apply (see OpArgs::geo)
-  float* geo32 = nullptr;
+  double* geo64 = nullptr;            // 2D: geometry table of the FP64 operator (see OpArgs::geo)
   void* cellbuf = nullptr;            // cell-wise results of the operator kernels (CellBuf), one buffer
   size_t cellbuf_bytes = 0;           // for all levels of a handle, on the handle's stream only
 };
@@ -51,8 +50,7 @@ cudaError_t launch_operator(const Level& lv, const Problem& pb, int mode, double
                             const T* state, const T* vprev, T* y, cudaStream_t stream,
                             int batch = 1, int64_t xs = 0, int64_t ys = 0);
 
-// y = rhs - J(state) x on a level (rhs null: y = J(state) x), the residual of a multigrid sweep;
-// one launch where the tiled 2D kernel applies, else the cell kernel and the node sums.
+// y = rhs - J(state) x on a level (rhs null: y = J(state) x), the residual of a multigrid sweep.
 // `columns` independent residuals at strides n_st (own rhs, x, state, y; per-column viscosity
 // nub[column] on the device, or null for pb.nu).
 template <typename T>
@@ -74,8 +72,7 @@ inline size_t cellbuf_need(int d, int n, int r, int k) {
 
 cudaError_t launch_initial_condition(const Level& lv, const Problem& pb, double* V0, cudaStream_t s);
 
-// Fill lv.geo64 / lv.geo32 (allocated by the caller: cells x 5 x (r+2)^2 entries each) for a 2D
-// level.
+// Fill lv.geo64 (allocated by the caller: cells x 5 x (r+2)^2 entries) of a 2D level.
 cudaError_t build_geometry(const Level& lv, const Problem& pb, cudaStream_t s);
 
 }  // namespace stmg

@@ -17,8 +17,6 @@ cudaError_t launch_operator<double>(const Level& lv, const Problem& pb, int mode
 template <>
 cudaError_t launch_level_residual<double>(const Level& lv, const Problem& pb, const double* rhs, const double* x,
                                        const double* state, double* y, cudaStream_t s, int columns, const double* nub) {
-  cudaError_t e = launch_jac_tiled<double>(lv, pb, x, state, rhs, y, s, columns, nub);
-  if (e != cudaErrorNotSupported) return e;
   return launch_any<double, MJ>(lv, pb, 0.0, x, state, nullptr, y, s, columns, lv.Nst, lv.Nst, lv.Nst, nub, rhs);
 }
 
@@ -69,10 +67,10 @@ static void geo_launch(const Level& lv, const Problem& pb, T* geo, cudaStream_t 
 }
 
 cudaError_t build_geometry(const Level& lv, const Problem& pb, cudaStream_t s) {
-  if (lv.d != 2 || !lv.geo64 || !lv.geo32) return cudaErrorInvalidValue;
+  if (lv.d != 2 || !lv.geo64) return cudaErrorInvalidValue;
   const int N = lv.r + 2;
-#define STMG_G(NN) { geo_launch<double, NN>(lv, pb, lv.geo64, s); geo_launch<float, NN>(lv, pb, lv.geo32, s); }
-  if (N == 3) STMG_G(3) else if (N == 4) STMG_G(4) else if (N == 5) STMG_G(5) else return cudaErrorInvalidValue;
+#define STMG_G(NN) geo_launch<double, NN>(lv, pb, lv.geo64, s);
+  if (N == 3) { STMG_G(3) } else if (N == 4) { STMG_G(4) } else if (N == 5) { STMG_G(5) } else { return cudaErrorInvalidValue; }
 #undef STMG_G
   return cudaGetLastError();
 }

@@ -4,10 +4,7 @@
 #include "level.hpp"
 #include "operator.cuh"
 #include "operator_cells.cuh"
-#include "operator2d_tile.cuh"
 #include "counters.hpp"
-#include <cstdlib>
-#include <cstring>
 
 namespace stmg {
 
@@ -82,14 +79,16 @@ static cudaError_t launch_dn(const Level& lv, const Problem& pb, double t0, cons
                              int batch, int64_t xs, int64_t ys, int64_t ss, const T* nub, const T* rhs) {
   constexpr int TPG = D == 2 ? N : N * N;             // threads per (cell, time node)
   constexpr bool F64 = sizeof(T) == 8;
-  constexpr int BT = D == 3 && (N == 5 || !F64) ? 256 : 192;
-  constexpr int MINB = D == 2 ? (F64 ? 2 : 4) : (F64 && N == 5 ? 1 : 2);
+  // threads per block and blocks per SM, as measured: 2D FP32 at 256^2 Q3/P2 DG(2) 128 x 7 53.3 us,
+  // 192 x 5 54.5, 192 x 4 57.4, 256 x 3 57.7, 192 x 3 64.0; 2D FP64 there 128 x 4 879 us, 96 x 4 882, 192 x 2
+  // 893, 256 x 1 981; 3D FP32 at 37^3 Q3/P2 DG(1) 128 x 4 284 us, 256 x 2 291, 128 x 5 297, 192 x 2 307; 3D
+  // FP64 at 64^3 Q2/P1 DG(2) 192 x 2 12.6 ms, 128 x 3 14.0 (more lanes idle)
+  constexpr int BT = D == 2 ? 128 : (N == 5 ? 256 : (F64 ? 192 : 128));
+  constexpr int MINB = D == 2 ? (F64 ? 4 : 7) : (N == 5 ? (F64 ? 1 : 2) : (F64 ? 2 : 4));
   const int kp1 = lv.k + 1;
   const Tab<T> tb = make_tab<T>(lv.tabs, pb.tau);
   const T* geo = nullptr;
-  if constexpr (D == 2) {
-    if constexpr (F64) geo = lv.geo64; else geo = lv.geo32;
-  }
+  if constexpr (D == 2 && F64) geo = lv.geo64;
   const int64_t cplane = D == 2 ? lv.n : (int64_t)lv.n * lv.n;   // cells per plane of the last axis
   CellBuf<T> cb{};
   int64_t cols;
@@ -119,47 +118,6 @@ static cudaError_t launch_dn(const Level& lv, const Problem& pb, double t0, cons
     }
   }
   return cudaGetLastError();
-}
-
-// Process-wide choice of the 2D FP32 Jacobian-apply kernel: the tiled single-launch kernel where it
-// applies (default), or the cell kernel with node sums when the environment variable STMG_APPLY2D
-// is "colour" (kept for comparisons; read once).
-inline bool apply2d_tiled() {
-  static const bool on = [] {
-    const char* v = std::getenv("STMG_APPLY2D");
-    return !(v && std::strcmp(v, "colour") == 0);
-  }();
-  return on;
-}
-
-template <typename T, int N>
-static cudaError_t jac_tiled_n(const Level& lv, const Problem& pb, const T* x, const T* state, const T* rhs, T* y,
-                               cudaStream_t s, int columns, const T* nub) {
-  OpArgs<T> A{level_args<T>(lv, pb, 0.0), x, state, nullptr, y, lv.Nst, lv.Nst, nullptr, lv.Nst, nub};
-  const Tab<T> tb = make_tab<T>(lv.tabs, pb.tau);
-  cudaError_t e = cudaErrorNotSupported;
-  if (lv.k == 0) e = launch_apply2d_tile<T, N, 1>(A, tb, rhs, lv.n, s, columns);
-  else if (lv.k == 1) e = launch_apply2d_tile<T, N, 2>(A, tb, rhs, lv.n, s, columns);
-  else if (lv.k == 2) e = launch_apply2d_tile<T, N, 3>(A, tb, rhs, lv.n, s, columns);
-  if (e == cudaSuccess) note_launch();
-  return e;
-}
-
-// y = J(state) x, or y = rhs - J(state) x when rhs is not null, by the tiled 2D kernel (one
-// launch, y written without a zero fill).  `columns` independent applies at strides n_st (own
-// increment, state, output and, with nub, viscosity).  cudaErrorNotSupported where it does not
-// apply (3D, Q4/P3, FP64, or the cell kernels chosen).
-template <typename T>
-cudaError_t launch_jac_tiled(const Level& lv, const Problem& pb, const T* x, const T* state, const T* rhs, T* y,
-                             cudaStream_t s, int columns = 1, const T* nub = nullptr) {
-  if constexpr (!std::is_same<T, float>::value) {
-    return cudaErrorNotSupported;
-  } else {
-    if (lv.d != 2 || !apply2d_tiled()) return cudaErrorNotSupported;
-    if (lv.r == 1) return jac_tiled_n<T, 3>(lv, pb, x, state, rhs, y, s, columns, nub);
-    if (lv.r == 2) return jac_tiled_n<T, 4>(lv, pb, x, state, rhs, y, s, columns, nub);
-    return cudaErrorNotSupported;
-  }
 }
 
 template <typename T, int MODE>

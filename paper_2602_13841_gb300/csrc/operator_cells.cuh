@@ -30,9 +30,12 @@
 // What bounds it: FP64 the FP64 pipe (2 multiply-adds per clock and SM; 84 % busy on 3D Q2/P1), FP32
 // shared-memory wavefronts and instruction issue.  Measured against the colour-by-colour kernels this
 // replaces (a zero fill, then a volume and a face launch per colour with one thread per point):
-//   3D 64^3 Q2/P1 DG(2) FP64 apply 20.14 -> 12.60 ms    3D 37^3 Q3/P2 DG(1) FP32 apply 940 -> 319 us
-//   3D 16^3 Q3/P2 DG(2) residual    3.00 -> 0.74 ms     2D 256^2 Q3/P2 DG(2) FP64 apply 1086 -> 900 us
-//   2D 8^2 Q2/P1 DG(1) FP64 apply    133 -> 37 us
+//   3D 64^3 Q2/P1 DG(2) FP64 apply 20.14 -> 12.63 ms    3D 37^3 Q3/P2 DG(1) FP32 apply 940 -> 284 us
+//   3D 16^3 Q3/P2 DG(2) residual    3.00 -> 0.73 ms     2D 256^2 Q3/P2 DG(2) FP64 apply 1086 -> 879 us
+//   2D 8^2 Q2/P1 DG(1) FP64 apply    133 -> 35 us
+// and, 2D FP32, against one kernel with a thread per cell on a tile of 16 x 8 cells in shared memory:
+//   256^2 Q3/P2 DG(2) 104 -> 51 us, Q2/P1 DG(1) 28.6 -> 22.7 us; 32^2 59 -> 8.8 us and 14.5 -> 8.0 us
+//   (Q2/P1 DG(0) alone is level: 14.1 -> 15.0 us at 256^2, 8.3 -> 8.2 us at 128^2)
 #pragma once
 #include <type_traits>
 
@@ -50,7 +53,7 @@ struct OpArgs {
   const T* vprev;    // R: V_{n-1}
   T* y;              // output
   int64_t xs, ys;    // batch strides (blockIdx.y selects the column of a batched apply)
-  const T* geo;      // 2D: per cell [5][Q] inverse Jacobian G[0][0], G[0][1], G[1][0], G[1][1] and
+  const T* geo;      // 2D FP64: per cell [5][Q] inverse Jacobian G[0][0], G[0][1], G[1][0], G[1][1] and
                      // JxW at the quadrature points (precomputed at set-up)
   int64_t ss;        // batch stride of the state (0: one state shared by the batch)
   const T* nub;      // per-batch-column viscosity (device, blockIdx.y), or null: L.nu
@@ -217,14 +220,21 @@ __device__ __forceinline__ void row_st(T* s, const T (&v)[N]) {
 template <int N> __host__ __device__ constexpr int plane3() { return N == 4 ? 20 : N * N; }
 template <int N> __host__ __device__ constexpr int arr3() { return plane3<N>() * N; }
 template <int N> __host__ __device__ constexpr int even4(int e) { return (e + 3) & ~3; }
-// One group's part of the 3D buffers: three arrays of values (B0), two times three of derivatives /
-// fluxes (B1, B2), pressure modes, a reduction line.  N = 4: 16 entries past a multiple of 32, so
-// that the two groups of a warp use different halves of the banks.
-template <int N> __host__ __device__ constexpr int group3() {
-  int e = even4<N>(9 * arr3<N>() + MAXNP + N * N);
-  if (N == 4)
-    while (e % 32 != 16) e += 4;
+// Smallest stride >= e that is `want` mod 32: neighbouring groups of a warp, `stride` entries apart, then
+// use different banks for their lines along every axis (with a stride of a multiple of 32 the lines of
+// 2D Q2/P1 collided: 256^2 Q2/P1 DG(2) FP32 apply 88 us instead of 35).
+__host__ __device__ constexpr int bank_stride(int e, int want) {
+  while (e % 32 != want) ++e;
   return e;
+}
+// One group's part of the 3D buffers: three arrays of values (B0), two times three of derivatives /
+// fluxes (B1, B2), pressure modes, a reduction line.
+template <int N> __host__ __device__ constexpr int group3() {
+  return bank_stride(9 * arr3<N>() + MAXNP + N * N, N == 3 ? 27 : (N == 4 ? 16 : 13));
+}
+// 2D: values, derivatives / fluxes, a reduction line, face arrays, pressure modes.
+template <int N> __host__ __device__ constexpr int group2() {
+  return bank_stride(4 * N * N + 13 * N + MAXNP, N == 3 ? 9 : (N == 4 ? 20 : 25));
 }
 
 template <typename T, int N, int MODE>
@@ -235,9 +245,13 @@ __host__ __device__ inline size_t cells3d_smem(int cpb, int kp1) {
 }
 template <typename T, int N>
 __host__ __device__ inline size_t cells2d_smem(int cpb, int kp1) {
-  constexpr int Q = N * N;
-  return sizeof(T) * ((size_t)cpb * kp1 * even4<N>(4 * Q + 13 * N + MAXNP) + 2 * MAXN * MAXN + MAXN * 4 + 2 * MAXN);
+  return sizeof(T) * ((size_t)cpb * kp1 * group2<N>() + 2 * MAXN * MAXN + MAXN * 4 + 2 * MAXN);
 }
+
+template <typename T>
+__device__ __forceinline__ T rcp_t(T v) { return (T)1 / v; }
+template <>
+__device__ __forceinline__ float rcp_t<float>(float v) { return __fdividef(1.0f, v); }
 
 // Small lookup tables indexed by a thread's own point: copied to shared memory, since constant-bank
 // reads serialise over different addresses.
@@ -334,9 +348,9 @@ __device__ __forceinline__ void face3d(const OpArgs<T>& A, const Tab<T>& tb, con
     T len2 = 0;
 #pragma unroll
     for (int i = 0; i < 3; ++i) { nrm[i] = det * G[AX][i] * nh; len2 += nrm[i] * nrm[i]; }
-    const T dS = sqrt(len2);
+    const T dS = sqrt(len2), is = (T)1 / dS;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) nrm[i] /= dS;
+    for (int i = 0; i < 3; ++i) nrm[i] *= is;
     jf = dS * (lt.qw[u] * lt.qw[v]);
     red[p] = jf;
     if (RES)
@@ -388,7 +402,7 @@ __device__ __forceinline__ void face3d(const OpArgs<T>& A, const Tab<T>& tb, con
     static_for<NPC>([&](auto m) {
       fp += tb.Pend[side][Mode<3, decltype(m)::value>::deg(AX)] * lt.P1[u][Mode<3, decltype(m)::value>::deg(T1)] * lt.P1[v][Mode<3, decltype(m)::value>::deg(T2)] * pm[decltype(m)::value];
     });
-    const T h = vol / area * L.hscale;
+    const T rh = area / (vol * L.hscale);             // 1 / h_{Gamma_D}
     T ghat[3], dn[3];
 #pragma unroll
     for (int m = 0; m < 3; ++m) ghat[m] = G[m][0] * nrm[0] + G[m][1] * nrm[1] + G[m][2] * nrm[2];
@@ -419,7 +433,7 @@ __device__ __forceinline__ void face3d(const OpArgs<T>& A, const Tab<T>& tb, con
     const T en = ev[0] * nrm[0] + ev[1] * nrm[1] + ev[2] * nrm[2];
     const T gn = gd[0] * nrm[0] + gd[1] * nrm[1] + gd[2] * nrm[2];
     const T wJ = tb.w[a] * jf;
-    const T p1 = nu * L.gamma1 / h, p2 = L.gamma2 / h;
+    const T p1 = nu * L.gamma1 * rh, p2 = L.gamma2 * rh;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       T t = -nu * dn[c] + p1 * ev[c] + p2 * en * nrm[c] + fp * nrm[c];
@@ -913,9 +927,9 @@ __device__ __forceinline__ void face2d(const OpArgs<T>& A, const Tab<T>& tb, con
     const T nh = side ? (T)1 : (T)-1;
     nrm[0] = det * G[AX][0] * nh;
     nrm[1] = det * G[AX][1] * nh;
-    const T dS = sqrt(nrm[0] * nrm[0] + nrm[1] * nrm[1]);
-    nrm[0] /= dS;
-    nrm[1] /= dS;
+    const T dS = sqrt(nrm[0] * nrm[0] + nrm[1] * nrm[1]), is = (T)1 / dS;
+    nrm[0] *= is;
+    nrm[1] *= is;
     jf = dS * lt.qw[u];
     red[u] = jf;
     if (RES)
@@ -942,7 +956,7 @@ __device__ __forceinline__ void face2d(const OpArgs<T>& A, const Tab<T>& tb, con
     if (RES) { fs[0] = fv[0]; fs[1] = fv[1]; }
     T fp = 0;
     static_for<NPC>([&](auto m) { fp += tb.Pend[side][Mode<2, decltype(m)::value>::deg(AX)] * lt.P1[u][Mode<2, decltype(m)::value>::deg(TX)] * pm[decltype(m)::value]; });
-    const T h = vol / area * L.hscale;
+    const T rh = area / (vol * L.hscale);             // 1 / h_{Gamma_D}
     T ghat[2], dn[2];
 #pragma unroll
     for (int m = 0; m < 2; ++m) ghat[m] = G[m][0] * nrm[0] + G[m][1] * nrm[1];
@@ -968,7 +982,7 @@ __device__ __forceinline__ void face2d(const OpArgs<T>& A, const Tab<T>& tb, con
     const T en = ev[0] * nrm[0] + ev[1] * nrm[1];
     const T gn = gd[0] * nrm[0] + gd[1] * nrm[1];
     const T wJ = tb.w[a] * jf;
-    const T p1 = nu * L.gamma1 / h, p2 = L.gamma2 / h;
+    const T p1 = nu * L.gamma1 * rh, p2 = L.gamma2 * rh;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       T t = -nu * dn[c] + p1 * ev[c] + p2 * en * nrm[c] + fp * nrm[c];
@@ -1008,7 +1022,7 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
                                                       int64_t c0, int64_t c1, int cpb, const T* __restrict__ rhs) {
   constexpr bool RES = MODE == MR, MASS = MODE == MM, JAC = MODE == MJ;
   constexpr int Q = N * N, NPC = npress<2, N>();
-  constexpr int GS = even4<N>(4 * Q + 13 * N + MAXNP);
+  constexpr int GS = group2<N>();
   const LevelArgs<T>& L = A.L;
   const int kp1 = tb.k + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1036,6 +1050,37 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
   const int64_t nbase = (int64_t)cc[0] * (N - 1) + n1 * ((int64_t)cc[1] * (N - 1));
   const int64_t poff = (int64_t)kp1 * L.Nv;
   const T wa = tb.w[a];
+  // the bilinear map x_l = mp[l][0] + mp[l][1] X + mp[l][2] Y + mp[l][3] XY.  FP32 evaluates its Jacobian
+  // at every point (a dozen operations against five loads of a table); FP64 reads the level's table,
+  // since every operation on its pipe counts, and needs the map on the boundary only.
+  constexpr bool TABLE = sizeof(T) == 8;
+  const bool bnd = !MASS && on && (cc[0] == 0 || cc[1] == 0 || cc[0] == L.n - 1 || cc[1] == L.n - 1);
+  T mp[2][4] = {{0, 1, 0, 0}, {0, 0, 1, 0}};
+  if (TABLE ? bnd : on) {
+    const int64_t v0 = (int64_t)cc[0] + (int64_t)(L.n + 1) * cc[1];
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      const T q0 = L.verts[2 * v0 + l], q1 = L.verts[2 * v0 + 2 + l];
+      const T q2 = L.verts[2 * (v0 + L.n + 1) + l], q3 = L.verts[2 * (v0 + L.n + 2) + l];
+      mp[l][0] = q0; mp[l][1] = q1 - q0; mp[l][2] = q2 - q0; mp[l][3] = (q3 - q2) - (q1 - q0);
+    }
+  }
+  // G (row-major) and JxW at the Gauss point (i, u)
+  const T* geo = TABLE ? A.geo + cell * 5 * Q + N * u : nullptr;
+  const auto geometry = [&](int i, T (&G)[4]) -> T {
+    if constexpr (TABLE) {
+#pragma unroll
+      for (int x = 0; x < 4; ++x) G[x] = geo[x * Q + i];
+      return geo[4 * Q + i];
+    } else {
+      const T X = tb.qx[i], Y = lt.qx[u];
+      const T J00 = mp[0][1] + mp[0][3] * Y, J01 = mp[0][2] + mp[0][3] * X;
+      const T J10 = mp[1][1] + mp[1][3] * Y, J11 = mp[1][2] + mp[1][3] * X;
+      const T det = J00 * J11 - J01 * J10, id = rcp_t<T>(det);
+      G[0] = J11 * id; G[1] = -J01 * id; G[2] = -J10 * id; G[3] = J00 * id;
+      return det * (tb.qw[i] * lt.qw[u]);
+    }
+  };
   // ---- nodal lines along y
   if (on) {
 #pragma unroll
@@ -1064,27 +1109,27 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
   if (on) {
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      line_ld<T, N>(B0 + c * Q + N * u, 1, xq[c]);
+      row_ld<T, N>(B0 + c * Q + N * u, xq[c]);
       line_B<T, N, false>(tb, xq[c]);
-      line_st<T, N>(B0 + c * Q + N * u, 1, xq[c]);
+      row_st<T, N>(B0 + c * Q + N * u, xq[c]);
       if (JAC) {
-        line_ld<T, N>(B1 + c * Q + N * u, 1, sq[c]);
+        row_ld<T, N>(B1 + c * Q + N * u, sq[c]);
         line_B<T, N, false>(tb, sq[c]);
       } else if (RES) {
         // V_{n-1}: group 0 interpolated it along y; every time node takes it from there
-        line_ld<T, N>(B0 - a * GS + 2 * Q + c * Q + N * u, 1, sq[c]);
+        row_ld<T, N>(B0 - a * GS + 2 * Q + c * Q + N * u, sq[c]);
         line_B<T, N, false>(tb, sq[c]);
       }
     }
     static_for<NPC>([&](auto m) { cx[Mode<2, decltype(m)::value>::deg(0)] += lt.P1[u][Mode<2, decltype(m)::value>::deg(1)] * s_pm[decltype(m)::value]; });
   }
   __syncthreads();
-  const T* geo = A.geo + cell * 5 * Q + N * u;
   if (on) {
     if (MASS) {
 #pragma unroll
       for (int i = 0; i < N; ++i) {
-        const T w = wa * geo[4 * Q + i];
+        T G[4];
+        const T w = wa * geometry(i, G);
         z[0][i] = w * xq[0][i];
         z[1][i] = w * xq[1][i];
         T pq = 0;
@@ -1127,7 +1172,8 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
       }
 #pragma unroll
       for (int i = 0; i < N; ++i) {
-        const T G00 = geo[i], G01 = geo[Q + i], G10 = geo[2 * Q + i], G11 = geo[3 * Q + i], jw = geo[4 * Q + i];
+        T G[4];
+        const T jw = geometry(i, G), G00 = G[0], G01 = G[1], G10 = G[2], G11 = G[3];
         T gp[2][2];
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
@@ -1205,7 +1251,7 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       line_B<T, N, true>(tb, z[c]);
-      line_st<T, N>(S + c * Q + N * u, 1, z[c]);
+      row_st<T, N>(S + c * Q + N * u, z[c]);
     }
   }
   __syncthreads();
@@ -1219,20 +1265,14 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
   T pp[NPC];
   static_for<NPC>([&](auto m) { pp[decltype(m)::value] = on ? lt.P1[u][Mode<2, decltype(m)::value>::deg(1)] * tx[Mode<2, decltype(m)::value>::deg(0)] : (T)0; });
   if (!MASS) {
-    const bool bnd = on && (cc[0] == 0 || cc[1] == 0 || cc[0] == L.n - 1 || cc[1] == L.n - 1);
     if (__syncthreads_or(bnd)) {
-      T vol = 0, mp[2][4] = {{0, 1, 0, 0}, {0, 0, 1, 0}};
+      T vol = 0;
       if (bnd) {
 #pragma unroll
         for (int c = 0; c < 2; ++c) line_st<T, N>(S + c * Q + u, N, z[c]);
-        const int64_t v0 = (int64_t)cc[0] + (int64_t)(L.n + 1) * cc[1];
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-          const T q0 = L.verts[2 * v0 + l], q1 = L.verts[2 * v0 + 2 + l];
-          const T q2 = L.verts[2 * (v0 + L.n + 1) + l], q3 = L.verts[2 * (v0 + L.n + 2) + l];
-          mp[l][0] = q0; mp[l][1] = q1 - q0; mp[l][2] = q2 - q0; mp[l][3] = (q3 - q2) - (q1 - q0);
-        }
-        for (int t = 0; t < Q; ++t) vol += A.geo[cell * 5 * Q + 4 * Q + t];
+        // |K|: det J of the bilinear map at the centre
+        vol = (mp[0][1] + (T)0.5 * mp[0][3]) * (mp[1][2] + (T)0.5 * mp[1][3]) -
+              (mp[0][2] + (T)0.5 * mp[0][3]) * (mp[1][1] + (T)0.5 * mp[1][3]);
       }
       // D at the lane's own point replaces Dc in the lane table: the faces differentiate nodal values
       for (int e = threadIdx.x; e < MAXN * MAXN; e += blockDim.x) lt.Dc[e / MAXN][e % MAXN] = tb.D[e / MAXN][e % MAXN];
@@ -1335,7 +1375,7 @@ __global__ void k_node_sum(CellBuf<T> cb, const T* src, T* y, T alpha, int n, in
   }
 }
 
-// Geometry table of a 2D level: per cell and Gauss point t the inverse Jacobian G (dxhat_m/dx_l)
+// Geometry table (FP64) of a 2D level: per cell and Gauss point t the inverse Jacobian G (dxhat_m/dx_l)
 // and JxW of the multilinear map.
 template <typename T, int N>
 __global__ void k_geo2d(LevelArgs<T> L, Tab<T> tb, T* __restrict__ geo, int64_t ncells) {

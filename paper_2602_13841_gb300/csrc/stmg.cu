@@ -101,10 +101,9 @@ static void build_level(Handle* h, Level& lv, const std::vector<double>& verts) 
     }
   }
   if (lv.d == 2) {
-    // geometry table of the 2D Jacobian apply (5 values per cell and Gauss point, both precisions)
+    // geometry table of the 2D FP64 operator (5 values per cell and Gauss point)
     const size_t ng = (size_t)ncells * 5 * (lv.r + 2) * (lv.r + 2);
     lv.geo64 = (double*)h->dalloc(ng * sizeof(double));
-    lv.geo32 = (float*)h->dalloc(ng * sizeof(float));
     if (build_geometry(lv, h->pb, h->stream) != cudaSuccess) throw CudaFailure(cudaErrorLaunchFailure);
   }
 }
@@ -168,7 +167,7 @@ stmg_status stmg_footprint(const stmg_params* p, uint64_t* bytes) {
     nst[l] = (lk + 1.0) * (Nv + Np);
     tot += 12.0 * d * std::pow(ln + 1.0, d);                            // vertices
     cbuf = std::max(cbuf, (double)cellbuf_need(d, ln, lr, lk));
-    if (d == 2) tot += cells * 5.0 * (lr + 2.0) * (lr + 2.0) * 12.0;    // 2D geometry tables
+    if (d == 2) tot += cells * 5.0 * (lr + 2.0) * (lr + 2.0) * 8.0;     // 2D geometry table
     tot += 5.0 * nst[l] * es;                                            // level vectors
     if (l + 1 < lv.size()) {
       double nl = std::pow(lr + 2.0, d), mv = d * nl, msp = mv + npc;
