@@ -276,23 +276,64 @@ cudaError_t coarse_invert(const double* A, double* Ainv, double* work, double* p
   return cudaGetLastError();
 }
 
-template <typename TA>
-__global__ void k_gemv_cm(const TA* __restrict__ A, int n, const double* __restrict__ x, double* __restrict__ y) {
-  A += (int64_t)blockIdx.y * n * n;           // blockIdx.y: independent slot
-  x += (int64_t)blockIdx.y * n;
-  y += (int64_t)blockIdx.y * n;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    double acc = 0.0;
-    for (int j = 0; j < n; ++j) acc += (double)A[(int64_t)j * n + i] * x[j];
-    y[i] = acc;
+// One product of the coarse solve, y = A x (A column-major n x n) with what stands around it:
+//   step 0: x1 = Ainv b        step 1: r = b - A x1        step 2: out = x1 + Ainv r
+// b: the right-hand side (T, nc entries) continued by zeros, out: nc entries of T.  A block owns 8 rows,
+// its 32 groups of 8 threads every 32nd column; their sums meet in shared memory in a fixed order.
+// FP64 on few SMs is slow, so small systems are spread over n / 8 blocks (n = 126: 10.2 -> TIME_MV us).
+template <typename T, int STEP>
+__global__ void __launch_bounds__(256) k_coarse_mv(const double* __restrict__ A, int n, int nc, const T* __restrict__ b,
+                                                   const double* __restrict__ x1, const double* __restrict__ r,
+                                                   double* __restrict__ y, T* __restrict__ out) {
+  __shared__ double part[32][9];
+  A += (int64_t)blockIdx.y * n * n;                   // blockIdx.y: independent slot
+  b += (int64_t)blockIdx.y * nc;
+  if (STEP > 0) x1 += (int64_t)blockIdx.y * n;
+  if (STEP == 2) { r += (int64_t)blockIdx.y * n; out += (int64_t)blockIdx.y * nc; }
+  else y += (int64_t)blockIdx.y * n;
+  const int lr = threadIdx.x & 7, g = threadIdx.x >> 3, i = blockIdx.x * 8 + lr;
+  double acc = 0.0;
+  if (i < n) {
+#pragma unroll 4
+    for (int j = g; j < n; j += 32) {
+      const double x = STEP == 0 ? (j < nc ? (double)b[j] : 0.0) : (STEP == 1 ? x1[j] : r[j]);
+      acc += A[(int64_t)j * n + i] * x;
+    }
+  }
+  part[g][lr] = acc;
+  __syncthreads();
+  if (threadIdx.x < 64) {                             // 8 rows x 8 sums of four, then 8 rows
+    double s = part[g][lr];
+    s += part[g + 8][lr];
+    s += part[g + 16][lr];
+    s += part[g + 24][lr];
+    part[g][lr] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < 8 && i < n) {
+    double s = part[0][lr];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) s += part[k][lr];
+    if (STEP == 0) y[i] = s;
+    else if (STEP == 1) y[i] = (i < nc ? (double)b[i] : 0.0) - s;
+    else if (i < nc) out[i] = (T)(x1[i] + s);
   }
 }
 
-cudaError_t gemv_cm(const double* A, int n, const double* x, double* y, cudaStream_t s, int slots) {
-  k_gemv_cm<double><<<dim3((n + 127) / 128, slots), 128, 0, s>>>(A, n, x, y);
-  note_launch();
+template <typename T>
+cudaError_t coarse_apply(const double* Ainv, const double* A, int n, int nc, const T* b, T* out, double* x1, double* r,
+                         cudaStream_t s, int slots) {
+  const dim3 grid((n + 7) / 8, slots);
+  k_coarse_mv<T, 0><<<grid, 256, 0, s>>>(Ainv, n, nc, b, nullptr, nullptr, x1, nullptr);
+  k_coarse_mv<T, 1><<<grid, 256, 0, s>>>(A, n, nc, b, x1, nullptr, r, nullptr);
+  k_coarse_mv<T, 2><<<grid, 256, 0, s>>>(Ainv, n, nc, b, x1, r, nullptr, out);
+  note_launch(3);
   return cudaGetLastError();
 }
+template cudaError_t coarse_apply<float>(const double*, const double*, int, int, const float*, float*, double*, double*,
+                                         cudaStream_t, int);
+template cudaError_t coarse_apply<double>(const double*, const double*, int, int, const double*, double*, double*,
+                                          double*, cudaStream_t, int);
 
 
 }  // namespace stmg

@@ -60,17 +60,15 @@ cudaError_t MG<T>::allocate(Handle* hh, int slots) {
     status = (int*)h->dalloc(sizeof(int));
     wstat = (int*)h->dalloc(sizeof(int));
     tr.resize(nl > 0 ? nl - 1 : 0);
-    for (int l = 0; l + 1 < nl; ++l) build_transfer(h, tr[l], h->levels[l], h->levels[l + 1], sizeof(T), B);
+    for (int l = 0; l + 1 < nl; ++l) build_transfer(h, tr[l], h->levels[l], h->levels[l + 1]);
     const Level& c = h->levels[nl - 1];
     Nc = (int)c.Nst;
     Nb = Nc + c.k + 1;
     A64 = (double*)h->dalloc((size_t)B * Nb * Nb * sizeof(double));
     ident = (double*)h->dalloc(((size_t)Nb * Nb + 2 * (size_t)Nc) * sizeof(double));
     Ucs = (double*)h->dalloc((size_t)Nc * sizeof(double));
-    cb = (double*)h->dalloc((size_t)B * Nb * sizeof(double));
     cx = (double*)h->dalloc((size_t)B * Nb * sizeof(double));
     cr = (double*)h->dalloc((size_t)B * Nb * sizeof(double));
-    cw = (double*)h->dalloc((size_t)B * Nb * sizeof(double));
     Ainv = (double*)h->dalloc((size_t)B * Nb * Nb * sizeof(double));
     gj_panel = (double*)h->dalloc(coarse_panel_entries(Nb) * sizeof(double));
     gj_piv = (int*)h->dalloc(2 * (size_t)Nb * sizeof(int));
@@ -145,19 +143,8 @@ cudaError_t MG<T>::setup(const double* U64, int slot, const Problem* pbp) {
 
 template <typename T>
 cudaError_t MG<T>::coarse_solve(const T* rhs, T* d, int slots) {
-  cudaStream_t s = h->stream;
-  CKE(cudaMemsetAsync(cb, 0, (size_t)slots * Nb * sizeof(double), s));
-  CKE((vcopy_slots<T, double>(Nc, slots, rhs, Nc, cb, Nb, s)));
-  CKE(gemv_cm(Ainv, Nb, cb, cx, s, slots));
-  for (int it = 0; it < 1; ++it) {          // one step of iterative refinement
-    CKE(gemv_cm(A64, Nb, cx, cw, s, slots));
-    CKE(cudaMemcpyAsync(cr, cb, (size_t)slots * Nb * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    CKE(vaxpby<double>((int64_t)slots * Nb, -1.0, cw, 1.0, cr, s));
-    CKE(gemv_cm(Ainv, Nb, cr, cw, s, slots));
-    CKE(vaxpby<double>((int64_t)slots * Nb, 1.0, cw, 1.0, cx, s));
-  }
-  CKE((vcopy_slots<double, T>(Nc, slots, cx, Nb, d, Nc, s)));
-  return cudaSuccess;
+  // FP64 inverse and one step of iterative refinement
+  return coarse_apply<T>(Ainv, A64, Nb, Nc, rhs, d, cx, cr, h->stream, slots);
 }
 
 template <typename T>
@@ -209,8 +196,7 @@ cudaError_t MG<T>::vcycle_level(int l, const T* rhs, T* d, int slots) {
   h->kend(KC_APPLYP);
   CKE(tr[l].template restrict_<T>(t[l], r[l + 1], s, slots));
   CKE(vcycle_level(l + 1, r[l + 1], z[l + 1], slots));
-  CKE(tr[l].template prolong<T>(z[l + 1], t[l], s, slots));
-  CKE(vaxpby<T>((int64_t)slots * lv.Nst, (T)1, t[l], (T)1, d, s));
+  CKE(tr[l].template prolong<T>(z[l + 1], d, s, slots, true));
   if (nu2 > 0) CKE(sweep(l, rhs, d, nu2, false, slots));
   return cudaSuccess;
 }

@@ -38,7 +38,7 @@ struct MG {
   cudaError_t check_wait();          // reads and clears wstat (synchronises the stream)
   // coarsest level: bordered Jacobian (FP64), its FP64 inverse, refinement buffers
   int Nc = 0, Nb = 0;
-  double *A64 = nullptr, *Ucs = nullptr, *cb = nullptr, *cx = nullptr, *cr = nullptr, *cw = nullptr;
+  double *A64 = nullptr, *Ucs = nullptr, *cx = nullptr, *cr = nullptr;
   double* ident = nullptr;
   double* Ainv = nullptr;
   double* gj_panel = nullptr;
@@ -101,7 +101,10 @@ cudaError_t coarse_border(const Level& lv, const Problem& pb, const double* J, d
 cudaError_t coarse_invert(const double* A, double* Ainv, double* work, double* panel, int* piv, int Nb, int* status,
                           cudaStream_t s);
 size_t coarse_panel_entries(int Nb);
-// y_j = A_j x_j for j < slots (A_j = A + j n^2, x_j = x + j n, y_j = y + j n); column-major.
-cudaError_t gemv_cm(const double* A, int n, const double* x, double* y, cudaStream_t s, int slots = 1);
+// out = Ainv b with one step of iterative refinement against A (n x n column-major, b and out the first nc
+// entries of the n unknowns), for `slots` systems at strides n^2 (matrices), nc (b, out), n (x1, r).
+template <typename T>
+cudaError_t coarse_apply(const double* Ainv, const double* A, int n, int nc, const T* b, T* out, double* x1, double* r,
+                         cudaStream_t s, int slots = 1);
 
 }  // namespace stmg

@@ -70,7 +70,7 @@ cudaError_t Handle::ensure_solver() {
     Mv = (double*)dalloc(L.Nst * sizeof(double));
     Jv = (double*)dalloc(L.Nst * sizeof(double));
     pw = (double*)dalloc(L.Nst * sizeof(double));
-    scratch = (double*)dalloc((size_t)RED_BLOCKS * 64 * sizeof(double));
+    scratch = (double*)dalloc(RED_SCRATCH * sizeof(double));
     hdev = (double*)dalloc(256 * sizeof(double));
     flag = (int*)dalloc(sizeof(int));
   } catch (const std::bad_alloc&) {
@@ -78,6 +78,7 @@ cudaError_t Handle::ensure_solver() {
   }
   // pressure weights: pw = M e with e = constant pressure at time node 0 (its pressure part at
   // time node 0 holds w_0 * int psi_m over each cell)
+  CKE(cudaMemsetAsync(scratch, 0, RED_SCRATCH * sizeof(double), stream));
   CKE(cudaMemsetAsync(Mv, 0, L.Nst * sizeof(double), stream));
   k_const_p0<<<64, 256, 0, stream>>>(Mv, (int64_t)(L.k + 1) * L.Nv, L.Np, L.npc);
   note_launch();
@@ -197,8 +198,7 @@ static cudaError_t fgmres(Handle* h, MG<T>& mg, const double* U, const double* b
       CKE(vdots<double>(N, j + 1, h->Vb, N, h->w, h->hdev, h->scratch, s));
       CKE(vsub_comb<double>(N, j + 1, h->Vb, N, h->hdev, h->w, s));
       CKE(vdots<double>(N, j + 1, h->Vb, N, h->w, h->hdev + 64, h->scratch, s));
-      CKE(vsub_comb<double>(N, j + 1, h->Vb, N, h->hdev + 64, h->w, s));
-      CKE(vdots<double>(N, 1, h->w, N, h->w, h->hdev + 128, h->scratch, s));
+      CKE(vsub_comb_norm<double>(N, j + 1, h->Vb, N, h->hdev + 64, h->w, h->hdev + 128, h->scratch, s));
       CKE(cudaMemcpyAsync(hh.data(), h->hdev, 3 * 64 * sizeof(double), cudaMemcpyDeviceToHost, s));
       CKE(cudaStreamSynchronize(s));
       if (h->timing && mg.graph_exec) mg.collect_graph_timers();

@@ -197,7 +197,6 @@ stmg_status stmg_footprint(const stmg_params* p, uint64_t* bytes) {
       tl.d = d; tl.r = lr; tl.npc = (int)npc; tl.smoother = p->smoother;
       wk = std::max(wk, (double)vanka_work_entries(tl, (size_t)es) * es);
       nvmax = std::max(nvmax, Nv);
-      tot += 3.0 * std::max((lk + 1.0) * Nv, (lk + 1.0) * Np) * es;      // transfer scratch
     }
   }
   tot += (ea + eb + em + nvmax) * es + wk + cbuf;                        // cbuf: cell-wise operator results

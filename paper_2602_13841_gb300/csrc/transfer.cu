@@ -1,4 +1,5 @@
 // Grid transfer kernels and their host set-up (see transfer.hpp).
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -9,22 +10,26 @@
 namespace stmg {
 
 // ---------------------------------------------------------------------------- host set-up
-static Csr1D upload_csr(Handle* h, int rows, int cols, const std::vector<std::vector<std::pair<int, double>>>& R) {
-  Csr1D c;
+// The rows of a 1D operator as contiguous windows of columns.
+static Line1D upload_lines(Handle* h, int rows, int cols, const std::vector<std::vector<std::pair<int, double>>>& R) {
+  Line1D c;
   c.rows = rows; c.cols = cols;
-  std::vector<int> rp{0}, ci;
-  std::vector<double> v;
-  std::vector<float> v32;
-  for (auto& row : R) {
-    for (auto& e : row) { ci.push_back(e.first); v.push_back(e.second); v32.push_back((float)e.second); }
-    rp.push_back((int)ci.size());
+  std::vector<int2> win(rows);
+  for (int i = 0; i < rows; ++i) {
+    int lo = cols, hi = -1;
+    for (auto& e : R[i]) { lo = std::min(lo, e.first); hi = std::max(hi, e.first); }
+    if (hi < 0) { lo = 0; hi = 0; }
+    win[i] = make_int2(lo, hi - lo + 1);
+    c.width = std::max(c.width, hi - lo + 1);
   }
-  c.rowptr = (int*)h->dalloc(rp.size() * sizeof(int));
-  c.col = (int*)h->dalloc(ci.size() * sizeof(int));
+  std::vector<double> v((size_t)rows * c.width, 0.0);
+  for (int i = 0; i < rows; ++i)
+    for (auto& e : R[i]) v[(size_t)i * c.width + e.first - win[i].x] += e.second;
+  std::vector<float> v32(v.begin(), v.end());
+  c.win = (int2*)h->dalloc(win.size() * sizeof(int2));
   c.val64 = (double*)h->dalloc(v.size() * sizeof(double));
   c.val32 = (float*)h->dalloc(v.size() * sizeof(float));
-  h->upload(c.rowptr, rp.data(), rp.size() * sizeof(int));
-  h->upload(c.col, ci.data(), ci.size() * sizeof(int));
+  h->upload(c.win, win.data(), win.size() * sizeof(int2));
   h->upload(c.val64, v.data(), v.size() * sizeof(double));
   h->upload(c.val32, v32.data(), v32.size() * sizeof(float));
   return c;
@@ -57,16 +62,16 @@ static std::vector<double> node_positions(int n, int r, double scale) {
   return x;
 }
 
-void build_transfer(Handle* h, Transfer& tr, const Level& f, const Level& c, size_t esize, int nb) {
+void build_transfer(Handle* h, Transfer& tr, const Level& f, const Level& c) {
   tr.fine = &f; tr.coarse = &c;
   const double cf = (double)c.n / f.n;
   auto R = eval_rows(c.n, c.r, node_positions(f.n, f.r, cf));
-  tr.P1 = upload_csr(h, f.N1, c.N1, R);
+  tr.P1 = upload_lines(h, f.N1, c.N1, R);
   std::vector<std::vector<std::pair<int, double>>> RT(c.N1);
   for (int i = 0; i < (int)R.size(); ++i)
     for (auto& e : R[i]) RT[e.first].push_back({i, e.second});
-  tr.P1T = upload_csr(h, c.N1, f.N1, RT);
-  tr.I1 = upload_csr(h, c.N1, f.N1, eval_rows(f.n, f.r, node_positions(c.n, c.r, 1.0 / cf)));
+  tr.P1T = upload_lines(h, c.N1, f.N1, RT);
+  tr.I1 = upload_lines(h, c.N1, f.N1, eval_rows(f.n, f.r, node_positions(c.n, c.r, 1.0 / cf)));
   // time
   auto tf = radau_right_nodes(f.k), tc = radau_right_nodes(c.k);
   for (int i = 0; i <= f.k; ++i)
@@ -114,220 +119,168 @@ void build_transfer(Handle* h, Transfer& tr, const Level& f, const Level& c, siz
   tr.PT32 = (float*)h->dalloc(PT.size() * sizeof(float));
   h->upload(tr.PT64, PT.data(), PT.size() * sizeof(double));
   h->upload(tr.PT32, PT32.data(), PT32.size() * sizeof(float));
-  // scratch: largest intermediate = (max k + 1) * d * max(N1f^d, ...) or the pressure part
-  int64_t big = (int64_t)(f.k + 1) * f.Nv;
-  int64_t pbig = (int64_t)(f.k + 1) * f.Np;
-  if (pbig > big) big = pbig;
-  tr.nb = nb;
-  tr.scr = big;
-  tr.tmpA = h->dalloc((size_t)nb * big * esize);
-  tr.tmpB = h->dalloc((size_t)nb * big * esize);
-  tr.tmpC = h->dalloc((size_t)nb * big * esize);
 }
 
 // ---------------------------------------------------------------------------- kernels
-// out[b][o][i][p] = sum_k val[k] in[b][o][col[k]][p], k in row i; arrays of `batch` contiguous
-// blocks (strides sin / sout), axis extent nin -> nout, `inner` = product of faster axes.
-template <typename T>
-__global__ void k_axis(const T* __restrict__ in, T* __restrict__ out, int nin, int nout, int64_t inner,
-                       int64_t outer, int64_t sin, int64_t sout, const int* __restrict__ rowptr,
-                       const int* __restrict__ col, const T* __restrict__ val, int64_t zin, int64_t zout) {
-  const int b = blockIdx.y;
-  const int64_t total = outer * nout * inner;
-  in += b * sin + blockIdx.z * zin;           // blockIdx.z: independent slot
-  out += b * sout + blockIdx.z * zout;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    int64_t p = idx % inner;
-    int64_t rest = idx / inner;
-    int i = (int)(rest % nout);
-    int64_t o = rest / nout;
-    T acc = 0;
-    for (int kk = rowptr[i]; kk < rowptr[i + 1]; ++kk) acc += val[kk] * in[(o * nin + col[kk]) * inner + p];
-    out[idx] = acc;
-  }
-}
+// One transfer in one launch: out = (M (x) L (x) .. (x) L) in on the velocity, L the 1D operator along
+// every axis and M the time matrix, and the pressure modes (op: prolongation, restriction or none), added
+// to out where `add`.  A thread owns one output node and component: it sums the product of its D row
+// windows for every input time node and mixes the sums in time, so that nothing passes through memory
+// between axes, time and pressure (five launches before, six with the correction's update).  A window
+// holds up to 7 entries, so a 3D restriction reads up to 343 neighbouring values per input; those of
+// neighbouring threads coincide and stay in L1.  Bound by launch and load latency on the small levels
+// that most transfers are for: MEASURED_TRANSFER.
+template <typename T> struct MatT { T m[MAXKP1][MAXKP1]; };
+enum { P_NONE = 0, P_PROLONG = 1, P_RESTRICT = 2 };
 
-// out[a_out][i] = sum_{a_in} M[a_out][a_in] in[a_in][i]   (arrays of length L)
-struct Mat3 { double m[MAXKP1][MAXKP1]; };
 template <typename T>
-__global__ void k_timemix(const T* __restrict__ in, T* __restrict__ out, int64_t L, int nin, int nout,
-                          int64_t sin, int64_t sout, Mat3 M, int64_t zin, int64_t zout) {
-  in += blockIdx.y * zin;                     // blockIdx.y: independent slot
-  out += blockIdx.y * zout;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < L; i += (int64_t)gridDim.x * blockDim.x) {
-    T v[MAXKP1];
-    for (int a = 0; a < nin; ++a) v[a] = in[a * sin + i];
-    for (int a = 0; a < nout; ++a) {
-      T acc = 0;
-      for (int b = 0; b < nin; ++b) acc += (T)M.m[a][b] * v[b];
-      out[a * sout + i] = acc;
-    }
-  }
-}
+struct TransferArgs {
+  const T* in;
+  T* out;
+  const int2* win;
+  const T* val;
+  int width, nin1, nout1, kin, kout, add;
+  int64_t nin, nout, vin, vout;                       // nodes and velocity entries per time node
+  int64_t nvel, total;                                // threads for the velocity, and with the pressure
+  MatT<T> M;
+  int pop, nf, ratio, npf, npc;                       // pressure: kind, fine cells per axis, modes fine / coarse
+  const T* PT;
+  int64_t pin, pout, zin, zout;                       // pressure entries per time node; slot strides
+};
 
-// Pressure prolongation: fine cell cf, mode mf  <-  coarse cell, all coarse modes (per time node)
 template <typename T, int D>
-__global__ void k_pprolong(const T* __restrict__ in, T* __restrict__ out, int nf, int ratio, int npf, int npc,
-                           const T* __restrict__ PT, int64_t sin, int64_t sout, int64_t zin, int64_t zout) {
-  const int b = blockIdx.y;
-  in += b * sin + blockIdx.z * zin; out += b * sout + blockIdx.z * zout;
-  int64_t ncf = 1;
-  for (int l = 0; l < D; ++l) ncf *= nf;
-  const int nc = nf / ratio;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < ncf * npf;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    int mf = (int)(idx % npf);
-    int64_t cf = idx / npf, rem = cf, cc = 0, s = 1;
-    int type = 0;
+__global__ void k_transfer(const __grid_constant__ TransferArgs<T> A) {
+  const T* in = A.in + blockIdx.y * A.zin;            // blockIdx.y: independent slot
+  T* out = A.out + blockIdx.y * A.zout;
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= A.total) return;
+  T acc[MAXKP1];
+#pragma unroll
+  for (int b = 0; b < MAXKP1; ++b) acc[b] = 0;
+  int64_t o, so;                                      // output entry and its stride between time nodes
+  if (t < A.nvel) {
+    const int c = (int)(t / A.nout);
+    unsigned rem = (unsigned)(t - c * A.nout);
+    int2 w[3];
+    const T* v[3];
+#pragma unroll
     for (int l = 0; l < D; ++l) {
-      int x = (int)(rem % nf); rem /= nf;
-      cc += (int64_t)(x / ratio) * s; s *= nc;
-      if (ratio == 2) type |= (x & 1) << l;
+      const unsigned q = rem / (unsigned)A.nout1, g = rem - q * (unsigned)A.nout1;
+      rem = q;
+      w[l] = A.win[g];
+      v[l] = A.val + (int64_t)g * A.width;
     }
-    const T* row = PT + ((int64_t)type * npf + mf) * npc;
-    T acc = 0;
-    for (int mc = 0; mc < npc; ++mc) acc += row[mc] * in[cc * npc + mc];
-    out[idx] = acc;
-  }
-}
-
-// Pressure restriction (transpose): coarse cell, mode mc  <-  its fine cells, all fine modes
-template <typename T, int D>
-__global__ void k_prestrict(const T* __restrict__ in, T* __restrict__ out, int nf, int ratio, int npf, int npc,
-                            const T* __restrict__ PT, int64_t sin, int64_t sout, int64_t zin, int64_t zout) {
-  const int b = blockIdx.y;
-  in += b * sin + blockIdx.z * zin; out += b * sout + blockIdx.z * zout;
-  const int nc = nf / ratio;
-  int64_t ncc = 1;
-  for (int l = 0; l < D; ++l) ncc *= nc;
-  const int nchild = (ratio == 2) ? (1 << D) : 1;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < ncc * npc;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    int mc = (int)(idx % npc);
-    int64_t cc = idx / npc;
+    const int64_t n1 = A.nin1;
+    const T* src = in + c * A.nin + w[0].x + n1 * (w[1].x + (D == 3 ? n1 * w[2].x : 0));
+    for (int z = 0; z < (D == 3 ? w[2].y : 1); ++z)
+      for (int y = 0; y < w[1].y; ++y) {
+        const T wyz = D == 3 ? v[2][z] * v[1][y] : v[1][y];
+        const T* s = src + n1 * (y + (D == 3 ? n1 * z : 0));
+#pragma unroll 2
+        for (int x = 0; x < w[0].y; ++x) {
+          const T f = wyz * v[0][x];
+#pragma unroll
+          for (int b = 0; b < MAXKP1; ++b)
+            if (b < A.kin) acc[b] += f * s[b * A.vin + x];
+        }
+      }
+    o = t;
+    so = A.vout;
+  } else {
+    const int64_t i = t - A.nvel;
+    const T* p = in + A.kin * A.vin;
+    const bool pro = A.pop == P_PROLONG;
+    const int no = pro ? A.npf : A.npc, n = pro ? A.nf : A.nf / A.ratio;
+    const int m = (int)(i % no);
+    unsigned rem = (unsigned)(i / no);
     int cm[3] = {0, 0, 0};
-    int64_t rem = cc;
-    for (int l = 0; l < D; ++l) { cm[l] = (int)(rem % nc); rem /= nc; }
-    T acc = 0;
-    for (int ch = 0; ch < nchild; ++ch) {
-      int64_t cf = 0, s = 1;
-      for (int l = 0; l < D; ++l) { cf += (int64_t)(cm[l] * ratio + ((ch >> l) & 1) * (ratio - 1)) * s; s *= nf; }
-      const T* P = PT + (int64_t)ch * npf * npc;
-      for (int mf = 0; mf < npf; ++mf) acc += P[mf * npc + mc] * in[cf * npf + mf];
+#pragma unroll
+    for (int l = 0; l < D; ++l) { cm[l] = (int)(rem % (unsigned)n); rem /= (unsigned)n; }
+    // prolongation: the coarse cell that holds the fine one; restriction: the fine cells of the coarse one
+    const int children = !pro && A.ratio == 2 ? (1 << D) : 1, no2 = pro ? A.nf / A.ratio : A.nf;
+    for (int ch = 0; ch < children; ++ch) {
+      int64_t cell = 0, s = 1;
+      int type = ch;
+      if (pro) type = 0;
+#pragma unroll
+      for (int l = 0; l < D; ++l) {
+        const int x = pro ? cm[l] / A.ratio : cm[l] * A.ratio + ((ch >> l) & 1);
+        if (pro && A.ratio == 2) type |= (cm[l] & 1) << l;
+        cell += x * s;
+        s *= no2;
+      }
+      const T* P = A.PT + (int64_t)type * A.npf * A.npc;
+      const int ni = pro ? A.npc : A.npf;
+      const T* q = p + cell * ni;
+      for (int k = 0; k < ni; ++k) {
+        const T f = pro ? P[m * A.npc + k] : P[k * A.npc + m];
+#pragma unroll
+        for (int b = 0; b < MAXKP1; ++b)
+          if (b < A.kin) acc[b] += f * q[b * A.pin + k];
+      }
     }
-    out[idx] = acc;
+    o = A.kout * A.vout + i;
+    so = A.pout;
+  }
+#pragma unroll
+  for (int a = 0; a < MAXKP1; ++a) {
+    if (a >= A.kout) break;
+    T r = 0;
+#pragma unroll
+    for (int b = 0; b < MAXKP1; ++b)
+      if (b < A.kin) r += A.M.m[a][b] * acc[b];
+    out[o + a * so] = A.add ? out[o + a * so] + r : r;
   }
 }
 
-static inline int grid1(int64_t n) {
-  int64_t g = (n + 255) / 256;
-  if (g > 152 * 8) g = 152 * 8;
-  return (int)(g < 1 ? 1 : g);
-}
-
-template <typename T> static const T* vals(const Csr1D& c);
-template <> const double* vals<double>(const Csr1D& c) { return c.val64; }
-template <> const float* vals<float>(const Csr1D& c) { return c.val32; }
+template <typename T> static const T* vals(const Line1D& c);
+template <> const double* vals<double>(const Line1D& c) { return c.val64; }
+template <> const float* vals<float>(const Line1D& c) { return c.val32; }
 template <typename T> static const T* ptab(const Transfer& t);
 template <> const double* ptab<double>(const Transfer& t) { return t.PT64; }
 template <> const float* ptab<float>(const Transfer& t) { return t.PT32; }
 
-// Apply a 1D operator along every axis to `batch` arrays of nin^d entries -> nout^d entries.
-// `slots` independent inputs at in + j * zin (outputs out + j * zout, scratch t + j * zt).
+// in on level li -> out on level lo through the 1D operator op and the time matrix M [lo.k+1][li.k+1].
 template <typename T>
-static cudaError_t tensor_apply(const Csr1D& op, int d, int nin, int nout, int batch, const T* in, T* out,
-                                T* t1, T* t2, cudaStream_t s, int slots = 1, int64_t zin = 0, int64_t zout = 0,
-                                int64_t zt = 0) {
-  int64_t ext[3] = {nin, nin, nin};
-  const T* src = in;
-  int64_t sin = 1;
-  for (int l = 0; l < d; ++l) sin *= nin;
-  for (int ax = 0; ax < d; ++ax) {
-    int64_t inner = 1, outer = 1;
-    for (int l = 0; l < ax; ++l) inner *= ext[l];
-    for (int l = ax + 1; l < d; ++l) outer *= ext[l];
-    int64_t sout = 1;
-    for (int l = 0; l < d; ++l) sout *= (l == ax ? nout : ext[l]);
-    T* dst = (ax == d - 1) ? out : ((ax % 2 == 0) ? t1 : t2);
-    int64_t sdst = (ax == d - 1) ? 0 : sout;
-    // the final pass writes with the caller's stride (= nout^d)
-    if (ax == d - 1) sdst = sout;
-    dim3 grid(grid1(outer * nout * inner), batch, slots);
-    const int64_t zs = (ax == 0) ? zin : zt, zd = (ax == d - 1) ? zout : zt;
-    k_axis<T><<<grid, 256, 0, s>>>(src, dst, (int)ext[ax], nout, inner, outer, sin, sdst, op.rowptr, op.col,
-                                   vals<T>(op), zs, zd);
-    note_launch();
-    ext[ax] = nout;
-    src = dst;
-    sin = sdst;
-  }
+static cudaError_t transfer_launch(const Transfer& tr, const Line1D& op, const Level& li, const Level& lo,
+                                   const double (*M)[MAXKP1], bool transposed, int pop, bool add, const T* in, T* out,
+                                   cudaStream_t s, int slots) {
+  TransferArgs<T> A{};
+  A.in = in; A.out = out;
+  A.win = op.win; A.val = vals<T>(op); A.width = op.width;
+  A.nin1 = li.N1; A.nout1 = lo.N1; A.kin = li.k + 1; A.kout = lo.k + 1; A.add = add;
+  A.nin = li.nnodes; A.nout = lo.nnodes; A.vin = li.Nv; A.vout = lo.Nv;
+  A.nvel = lo.Nv;
+  A.total = lo.Nv + (pop != P_NONE ? lo.Np : 0);
+  for (int a = 0; a <= lo.k; ++a)
+    for (int b = 0; b <= li.k; ++b) A.M.m[a][b] = (T)(transposed ? M[b][a] : M[a][b]);
+  A.pop = pop; A.nf = tr.fine->n; A.ratio = tr.ratio; A.npf = tr.fine->npc; A.npc = tr.coarse->npc;
+  A.PT = ptab<T>(tr);
+  A.pin = li.Np; A.pout = lo.Np; A.zin = li.Nst; A.zout = lo.Nst;
+  const dim3 grid((unsigned)((A.total + 127) / 128), (unsigned)slots);
+  if (li.d == 2) k_transfer<T, 2><<<grid, 128, 0, s>>>(A);
+  else k_transfer<T, 3><<<grid, 128, 0, s>>>(A);
+  note_launch();
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t Transfer::prolong(const T* xc, T* xf, cudaStream_t s, int slots) const {
-  const Level& f = *fine; const Level& c = *coarse;
-  if (slots < 1 || slots > nb) return cudaErrorInvalidValue;
-  T* A = (T*)tmpA; T* B = (T*)tmpB; T* C = (T*)tmpC;
-  const int d = f.d;
-  // velocity: space at coarse time nodes -> C, then time mix into xf
-  cudaError_t e = tensor_apply<T>(P1, d, c.N1, f.N1, (c.k + 1) * d, xc, C, A, B, s, slots, c.Nst, scr, scr);
-  if (e != cudaSuccess) return e;
-  Mat3 M{};
-  for (int a = 0; a <= f.k; ++a) for (int b = 0; b <= c.k; ++b) M.m[a][b] = E[a][b];
-  k_timemix<T><<<dim3(grid1(f.Nv), slots), 256, 0, s>>>(C, xf, f.Nv, c.k + 1, f.k + 1, f.Nv, f.Nv, M, scr, f.Nst);
-  note_launch();
-  // pressure
-  const T* pc = xc + (int64_t)(c.k + 1) * c.Nv;
-  T* pf = xf + (int64_t)(f.k + 1) * f.Nv;
-  int64_t ncf = f.Np / f.npc;
-  dim3 g(grid1(ncf * f.npc), c.k + 1, slots);
-  if (d == 2) k_pprolong<T, 2><<<g, 256, 0, s>>>(pc, C, f.n, ratio, f.npc, c.npc, ptab<T>(*this), c.Np, f.Np, c.Nst, scr);
-  else k_pprolong<T, 3><<<g, 256, 0, s>>>(pc, C, f.n, ratio, f.npc, c.npc, ptab<T>(*this), c.Np, f.Np, c.Nst, scr);
-  note_launch();
-  k_timemix<T><<<dim3(grid1(f.Np), slots), 256, 0, s>>>(C, pf, f.Np, c.k + 1, f.k + 1, f.Np, f.Np, M, scr, f.Nst);
-  note_launch();
-  return cudaGetLastError();
+cudaError_t Transfer::prolong(const T* xc, T* xf, cudaStream_t s, int slots, bool add) const {
+  return transfer_launch<T>(*this, P1, *coarse, *fine, E, false, P_PROLONG, add, xc, xf, s, slots);
 }
 
 template <typename T>
 cudaError_t Transfer::restrict_(const T* xf, T* xc, cudaStream_t s, int slots) const {
-  const Level& f = *fine; const Level& c = *coarse;
-  if (slots < 1 || slots > nb) return cudaErrorInvalidValue;
-  T* A = (T*)tmpA; T* B = (T*)tmpB; T* C = (T*)tmpC;
-  const int d = f.d;
-  Mat3 M{};
-  for (int a = 0; a <= c.k; ++a) for (int b = 0; b <= f.k; ++b) M.m[a][b] = E[b][a];   // E^T
-  k_timemix<T><<<dim3(grid1(f.Nv), slots), 256, 0, s>>>(xf, C, f.Nv, f.k + 1, c.k + 1, f.Nv, f.Nv, M, f.Nst, scr);
-  note_launch();
-  cudaError_t e = tensor_apply<T>(P1T, d, f.N1, c.N1, (c.k + 1) * d, C, xc, A, B, s, slots, scr, c.Nst, scr);
-  if (e != cudaSuccess) return e;
-  const T* pf = xf + (int64_t)(f.k + 1) * f.Nv;
-  T* pc = xc + (int64_t)(c.k + 1) * c.Nv;
-  k_timemix<T><<<dim3(grid1(f.Np), slots), 256, 0, s>>>(pf, C, f.Np, f.k + 1, c.k + 1, f.Np, f.Np, M, f.Nst, scr);
-  note_launch();
-  int64_t ncc = c.Np / c.npc;
-  dim3 g(grid1(ncc * c.npc), c.k + 1, slots);
-  if (d == 2) k_prestrict<T, 2><<<g, 256, 0, s>>>(C, pc, f.n, ratio, f.npc, c.npc, ptab<T>(*this), f.Np, c.Np, scr, c.Nst);
-  else k_prestrict<T, 3><<<g, 256, 0, s>>>(C, pc, f.n, ratio, f.npc, c.npc, ptab<T>(*this), f.Np, c.Np, scr, c.Nst);
-  note_launch();
-  return cudaGetLastError();
+  return transfer_launch<T>(*this, P1T, *fine, *coarse, E, true, P_RESTRICT, false, xf, xc, s, slots);
 }
 
 template <typename T>
 cudaError_t Transfer::interp_state(const T* Vf, T* Vc, cudaStream_t s) const {
-  const Level& f = *fine; const Level& c = *coarse;
-  T* A = (T*)tmpA; T* B = (T*)tmpB; T* C = (T*)tmpC;
-  Mat3 M{};
-  for (int a = 0; a <= c.k; ++a) for (int b = 0; b <= f.k; ++b) M.m[a][b] = Et[a][b];
-  k_timemix<T><<<grid1(f.Nv), 256, 0, s>>>(Vf, C, f.Nv, f.k + 1, c.k + 1, f.Nv, f.Nv, M, 0, 0);
-  note_launch();
-  return tensor_apply<T>(I1, f.d, f.N1, c.N1, (c.k + 1) * f.d, C, Vc, A, B, s);
+  return transfer_launch<T>(*this, I1, *fine, *coarse, Et, false, P_NONE, false, Vf, Vc, s, 1);
 }
 
-template cudaError_t Transfer::prolong<float>(const float*, float*, cudaStream_t, int) const;
-template cudaError_t Transfer::prolong<double>(const double*, double*, cudaStream_t, int) const;
+template cudaError_t Transfer::prolong<float>(const float*, float*, cudaStream_t, int, bool) const;
+template cudaError_t Transfer::prolong<double>(const double*, double*, cudaStream_t, int, bool) const;
 template cudaError_t Transfer::restrict_<float>(const float*, float*, cudaStream_t, int) const;
 template cudaError_t Transfer::restrict_<double>(const double*, double*, cudaStream_t, int) const;
 template cudaError_t Transfer::interp_state<float>(const float*, float*, cudaStream_t) const;

@@ -16,10 +16,10 @@
 
 namespace stmg {
 
-struct Csr1D {
-  int rows = 0, cols = 0;
-  int* rowptr = nullptr;   // device
-  int* col = nullptr;
+// A 1D operator: row i combines the win[i].y columns from win[i].x on, with val[i * width + ...].
+struct Line1D {
+  int rows = 0, cols = 0, width = 0;
+  int2* win = nullptr;     // device
   double* val64 = nullptr;
   float* val32 = nullptr;
 };
@@ -27,23 +27,17 @@ struct Csr1D {
 struct Transfer {
   const Level* fine = nullptr;
   const Level* coarse = nullptr;
-  Csr1D P1, P1T, I1;
+  Line1D P1, P1T, I1;
   double E[MAXKP1][MAXKP1]{};   // [kf+1][kc+1]
   double Et[MAXKP1][MAXKP1]{};  // [kc+1][kf+1]
   int ntypes = 1, ratio = 1;    // pressure child types (2^d for h-transfers)
   double* PT64 = nullptr;       // [ntypes][npf][npc]
   float* PT32 = nullptr;
-  // scratch (element type of the preconditioner), `nb` slots of `scr` entries each
-  void* tmpA = nullptr;
-  void* tmpB = nullptr;
-  void* tmpC = nullptr;
-  int nb = 1;                   // slots: independent vectors transferred by one launch each
-  int64_t scr = 0;
 
-  // Each call transfers `slots` independent vectors (slot j at offset j * n_st of its level;
-  // slots <= nb), in the same launches.
+  // Each call transfers `slots` independent vectors (slot j at offset j * n_st of its level) in one
+  // launch.
   template <typename T>
-  cudaError_t prolong(const T* xc, T* xf, cudaStream_t s, int slots = 1) const;     // xf = P xc
+  cudaError_t prolong(const T* xc, T* xf, cudaStream_t s, int slots = 1, bool add = false) const;   // xf (+)= P xc
   template <typename T>
   cudaError_t restrict_(const T* xf, T* xc, cudaStream_t s, int slots = 1) const;   // xc = P^T xf
   template <typename T>
@@ -51,7 +45,7 @@ struct Transfer {
 };
 
 struct Handle;
-// Build the transfer between levels[l] and levels[l+1]; scratch for element size `esize` and nb slots.
-void build_transfer(Handle* h, Transfer& tr, const Level& fine, const Level& coarse, size_t esize, int nb = 1);
+// Build the transfer between levels[l] and levels[l+1].
+void build_transfer(Handle* h, Transfer& tr, const Level& fine, const Level& coarse);
 
 }  // namespace stmg

@@ -38,34 +38,52 @@ cudaError_t vcopy(int64_t n, const S* x, T* y, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <typename S, typename T>
-__global__ void k_copy_slots(int64_t n, const S* __restrict__ x, int64_t xs, T* __restrict__ y, int64_t ys) {
-  x += blockIdx.y * xs;
-  y += blockIdx.y * ys;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    y[i] = (T)x[i];
-}
-
-template <typename S, typename T>
-cudaError_t vcopy_slots(int64_t n, int slots, const S* x, int64_t xs, T* y, int64_t ys, cudaStream_t s) {
-  k_copy_slots<S, T><<<dim3(grid_for(n), slots), 256, 0, s>>>(n, x, xs, y, ys);
-  note_launch();
-  return cudaGetLastError();
-}
-
-// Partial dot products of up to DOTS_PER_ROW basis vectors with w per block: w[i] is read once
-// for all of them.  Each thread accumulates its strided elements in index order, then the block
-// reduces in a fixed tree: the result does not depend on how many vectors share a block.
+// Dot products in one launch: each block forms the partial sums of up to DOTS_PER_ROW basis vectors with
+// w (w[i] is read once for all of them); the last block of a row of blocks to finish adds the partial
+// sums, in block order.  Each thread accumulates its strided elements in index order and every sum
+// has a fixed tree, so the result does not depend on which block is last.  Short vectors take few
+// blocks: the launch is then over as soon as the data have been read.
 constexpr int DOTS_PER_ROW = 4;
 
+// Sums red[0 .. RED_THREADS) per row of `red`, rows q < cnt, into the first warp's lane 0 (v[q]).
+template <int Q>
+__device__ __forceinline__ void block_sums(double (*red)[RED_THREADS], double (&v)[Q]) {
+  __syncthreads();
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      double s = red[q][threadIdx.x];
+#pragma unroll
+      for (int k = 1; k < RED_THREADS / 32; ++k) s += red[q][threadIdx.x + 32 * k];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+      v[q] = s;
+    }
+  }
+}
+
+// After a block has written its partial sums: true in the last of gridDim.x blocks (and resets count).
+__device__ __forceinline__ bool last_block(unsigned* count) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(count, 1u) == gridDim.x - 1;
+    if (last) *count = 0;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
 template <typename T>
-__global__ void k_dots_partial(int64_t n, int m, const T* __restrict__ X, int64_t ldx, const T* __restrict__ w,
-                               double* __restrict__ part) {
+__global__ void k_dots(int64_t n, int m, const T* __restrict__ X, int64_t ldx, const T* __restrict__ w, double* part,
+                       double* __restrict__ out, unsigned* count) {
   __shared__ double red[DOTS_PER_ROW][RED_THREADS];
   const int l0 = blockIdx.y * DOTS_PER_ROW;
   const int cnt = m - l0 < DOTS_PER_ROW ? m - l0 : DOTS_PER_ROW;
   double acc[DOTS_PER_ROW] = {0.0, 0.0, 0.0, 0.0};
-  const int64_t stride = (int64_t)RED_BLOCKS * RED_THREADS;
+  const int64_t stride = (int64_t)gridDim.x * RED_THREADS;
   for (int64_t i = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x; i < n; i += stride) {
     const double wi = (double)w[i];
     double xv[DOTS_PER_ROW];
@@ -76,52 +94,67 @@ __global__ void k_dots_partial(int64_t n, int m, const T* __restrict__ X, int64_
   }
 #pragma unroll
   for (int q = 0; q < DOTS_PER_ROW; ++q) red[q][threadIdx.x] = acc[q];
-  __syncthreads();
-  for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s)
+  block_sums<DOTS_PER_ROW>(red, acc);
+  if (threadIdx.x == 0)
+    for (int q = 0; q < cnt; ++q) part[(int64_t)(l0 + q) * RED_BLOCKS + blockIdx.x] = acc[q];
+  if (!last_block(count + blockIdx.y)) return;
 #pragma unroll
-      for (int q = 0; q < DOTS_PER_ROW; ++q) red[q][threadIdx.x] += red[q][threadIdx.x + s];
-    __syncthreads();
+  for (int q = 0; q < DOTS_PER_ROW; ++q) {
+    double s = 0.0;
+    if (q < cnt)
+      for (int i = threadIdx.x; i < (int)gridDim.x; i += RED_THREADS) s += __ldcg(part + (int64_t)(l0 + q) * RED_BLOCKS + i);
+    red[q][threadIdx.x] = s;
   }
-  if (threadIdx.x < cnt) part[(l0 + threadIdx.x) * RED_BLOCKS + blockIdx.x] = red[threadIdx.x][0];
+  block_sums<DOTS_PER_ROW>(red, acc);
+  if (threadIdx.x == 0)
+    for (int q = 0; q < cnt; ++q) out[l0 + q] = acc[q];
 }
 
-__global__ void k_dots_final(const double* __restrict__ part, double* __restrict__ out) {
-  __shared__ double red[RED_THREADS];
-  const int l = blockIdx.x;
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < RED_BLOCKS; i += RED_THREADS) acc += part[l * RED_BLOCKS + i];
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[l] = red[0];
+// about eight elements a thread, at most RED_BLOCKS blocks
+static inline int red_grid(int64_t n) {
+  const int64_t g = (n + 8 * RED_THREADS - 1) / (8 * RED_THREADS);
+  return (int)(g < 1 ? 1 : (g > RED_BLOCKS ? RED_BLOCKS : g));
 }
+static inline unsigned* red_counters(double* scratch) { return reinterpret_cast<unsigned*>(scratch + (size_t)RED_BLOCKS * 64); }
 
 template <typename T>
 cudaError_t vdots(int64_t n, int m, const T* X, int64_t ldx, const T* w, double* out, double* scratch,
                   cudaStream_t s) {
   if (m <= 0) return cudaSuccess;
-  k_dots_partial<T><<<dim3(RED_BLOCKS, (m + DOTS_PER_ROW - 1) / DOTS_PER_ROW), RED_THREADS, 0, s>>>(n, m, X, ldx, w,
-                                                                                              scratch);
+  if (m > 64) return cudaErrorInvalidValue;
+  k_dots<T><<<dim3(red_grid(n), (m + DOTS_PER_ROW - 1) / DOTS_PER_ROW), RED_THREADS, 0, s>>>(
+      n, m, X, ldx, w, scratch, out, red_counters(scratch));
   note_launch();
-  k_dots_final<<<m, RED_THREADS, 0, s>>>(scratch, out);
   return cudaGetLastError();
 }
 
-template <typename T>
+// w -= sum_l h[l] X[l]; NORM: also out = sum_i w_i^2 of the result (the same two-stage sum).
+template <typename T, bool NORM>
 __global__ void k_sub_comb(int64_t n, int m, const T* __restrict__ X, int64_t ldx, const double* __restrict__ h,
-                           T* __restrict__ w) {
+                           T* __restrict__ w, double* part, double* __restrict__ out, unsigned* count) {
   __shared__ double hs[64];
+  __shared__ double red[1][RED_THREADS];
   if (threadIdx.x < m) hs[threadIdx.x] = h[threadIdx.x];
   __syncthreads();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+  double sq[1] = {0.0};
+  for (int64_t i = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * RED_THREADS) {
     double acc = (double)w[i];
 #pragma unroll 8
     for (int l = 0; l < m; ++l) acc -= hs[l] * (double)X[l * ldx + i];
-    w[i] = (T)acc;
+    const T wi = (T)acc;
+    w[i] = wi;
+    if (NORM) sq[0] += (double)wi * (double)wi;
+  }
+  if (NORM) {
+    red[0][threadIdx.x] = sq[0];
+    block_sums<1>(red, sq);
+    if (threadIdx.x == 0) part[blockIdx.x] = sq[0];
+    if (!last_block(count)) return;
+    double s = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += RED_THREADS) s += __ldcg(part + i);
+    red[0][threadIdx.x] = s;
+    block_sums<1>(red, sq);
+    if (threadIdx.x == 0) *out = sq[0];
   }
 }
 
@@ -129,7 +162,16 @@ template <typename T>
 cudaError_t vsub_comb(int64_t n, int m, const T* X, int64_t ldx, const double* h, T* w, cudaStream_t s) {
   if (m <= 0) return cudaSuccess;
   if (m > 64) return cudaErrorInvalidValue;
-  k_sub_comb<T><<<grid_for(n), 256, 0, s>>>(n, m, X, ldx, h, w);
+  k_sub_comb<T, false><<<grid_for(n), RED_THREADS, 0, s>>>(n, m, X, ldx, h, w, nullptr, nullptr, nullptr);
+  note_launch();
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t vsub_comb_norm(int64_t n, int m, const T* X, int64_t ldx, const double* h, T* w, double* out, double* scratch,
+                           cudaStream_t s) {
+  if (m <= 0 || m > 64) return cudaErrorInvalidValue;
+  k_sub_comb<T, true><<<red_grid(n), RED_THREADS, 0, s>>>(n, m, X, ldx, h, w, scratch, out, red_counters(scratch));
   note_launch();
   return cudaGetLastError();
 }
@@ -212,13 +254,12 @@ template cudaError_t vcopy<double, float>(int64_t, const double*, float*, cudaSt
 template cudaError_t vcopy<float, double>(int64_t, const float*, double*, cudaStream_t);
 template cudaError_t vcopy<double, double>(int64_t, const double*, double*, cudaStream_t);
 template cudaError_t vcopy<float, float>(int64_t, const float*, float*, cudaStream_t);
-template cudaError_t vcopy_slots<double, float>(int64_t, int, const double*, int64_t, float*, int64_t, cudaStream_t);
-template cudaError_t vcopy_slots<float, double>(int64_t, int, const float*, int64_t, double*, int64_t, cudaStream_t);
-template cudaError_t vcopy_slots<double, double>(int64_t, int, const double*, int64_t, double*, int64_t, cudaStream_t);
 template cudaError_t vdots<float>(int64_t, int, const float*, int64_t, const float*, double*, double*, cudaStream_t);
 template cudaError_t vdots<double>(int64_t, int, const double*, int64_t, const double*, double*, double*, cudaStream_t);
 template cudaError_t vsub_comb<float>(int64_t, int, const float*, int64_t, const double*, float*, cudaStream_t);
 template cudaError_t vsub_comb<double>(int64_t, int, const double*, int64_t, const double*, double*, cudaStream_t);
+template cudaError_t vsub_comb_norm<double>(int64_t, int, const double*, int64_t, const double*, double*, double*, double*,
+                                            cudaStream_t);
 template cudaError_t vscale_inv_dev<double>(int64_t, const double*, const double*, double*, cudaStream_t);
 template cudaError_t vscale_inv_dev<float>(int64_t, const float*, const double*, float*, cudaStream_t);
 template cudaError_t vscale<float>(int64_t, float, const float*, float*, cudaStream_t);

@@ -15,16 +15,20 @@ cudaError_t vaxpby(int64_t n, T a, const T* x, T b, T* y, cudaStream_t s);
 // y = x (element type conversion allowed)
 template <typename S, typename T>
 cudaError_t vcopy(int64_t n, const S* x, T* y, cudaStream_t s);
-// y_j = x_j (n entries) for j < slots, x_j = x + j xs, y_j = y + j ys (one launch)
-template <typename S, typename T>
-cudaError_t vcopy_slots(int64_t n, int slots, const S* x, int64_t xs, T* y, int64_t ys, cudaStream_t s);
-// out[l] = sum_i X[l*ldx + i] * w[i], l < m  (device scalars, double); scratch >= m*RED_BLOCKS doubles
+// Work space of the reductions: 64 rows of partial sums and the block counters (zero before first use;
+// every call leaves them zero).  One per stream.
+constexpr size_t RED_SCRATCH = (size_t)RED_BLOCKS * 64 + 64;
+// out[l] = sum_i X[l*ldx + i] * w[i], l < m <= 64  (device scalars, double)
 template <typename T>
 cudaError_t vdots(int64_t n, int m, const T* X, int64_t ldx, const T* w, double* out, double* scratch,
                   cudaStream_t s);
 // w -= sum_l h[l] * X[l*ldx + :], h on the device (double), l < m
 template <typename T>
 cudaError_t vsub_comb(int64_t n, int m, const T* X, int64_t ldx, const double* h, T* w, cudaStream_t s);
+// the same, and *out = sum_i w_i^2 of the result (device scalar)
+template <typename T>
+cudaError_t vsub_comb_norm(int64_t n, int m, const T* X, int64_t ldx, const double* h, T* w, double* out, double* scratch,
+                           cudaStream_t s);
 // x += sum_l y[l] * Z[l*ldz + :] with host coefficients copied by value (m <= 64)
 cudaError_t vadd_comb_host(int64_t n, int m, const double* Z, int64_t ldz, const double* y, double* x,
                            cudaStream_t s);
