@@ -280,7 +280,7 @@ cudaError_t coarse_invert(const double* A, double* Ainv, double* work, double* p
 //   step 0: x1 = Ainv b        step 1: r = b - A x1        step 2: out = x1 + Ainv r
 // b: the right-hand side (T, nc entries) continued by zeros, out: nc entries of T.  A block owns 8 rows,
 // its 32 groups of 8 threads every 32nd column; their sums meet in shared memory in a fixed order.
-// FP64 on few SMs is slow, so small systems are spread over n / 8 blocks (n = 126: 10.2 -> TIME_MV us).
+// FP64 on few SMs is slow, so small systems are spread over n / 8 blocks (n = 126: 10.2 -> 3.7 us).
 template <typename T, int STEP>
 __global__ void __launch_bounds__(256) k_coarse_mv(const double* __restrict__ A, int n, int nc, const T* __restrict__ b,
                                                    const double* __restrict__ x1, const double* __restrict__ r,

@@ -1,5 +1,6 @@
 // Vector kernels (see vec.cuh).  Grid-stride loops sized as a multiple of the SM count;
 // reductions in a fixed order (block partial sums, then one block per result).
+#include <algorithm>
 #include "vec.cuh"
 #include "counters.hpp"
 
@@ -52,9 +53,15 @@ __device__ __forceinline__ void block_sums(double (*red)[RED_THREADS], double (&
   if (threadIdx.x < 32) {
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
-      double s = red[q][threadIdx.x];
+      // a tree: FP64 additions are slow one after another
+      double t[RED_THREADS / 32];
 #pragma unroll
-      for (int k = 1; k < RED_THREADS / 32; ++k) s += red[q][threadIdx.x + 32 * k];
+      for (int k = 0; k < RED_THREADS / 32; ++k) t[k] = red[q][threadIdx.x + 32 * k];
+#pragma unroll
+      for (int h = RED_THREADS / 64; h > 0; h >>= 1)
+#pragma unroll
+        for (int k = 0; k < h; ++k) t[k] += t[k + h];
+      double s = t[0];
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
       v[q] = s;
@@ -110,9 +117,12 @@ __global__ void k_dots(int64_t n, int m, const T* __restrict__ X, int64_t ldx, c
     for (int q = 0; q < cnt; ++q) out[l0 + q] = acc[q];
 }
 
-// about eight elements a thread, at most RED_BLOCKS blocks
+// Short vectors: two elements a thread, up to two blocks an SM (eight a thread left most SMs idle; 2D 32^2
+// Q2/P1 DG(1) slab solve 8.09 -> 7.87 ms).  Long ones: eight a thread, so that the last block has fewer partial
+// sums to add (two a thread throughout: 2D 128^2 Q3/P2 DG(2) slab solve 1-2 % slower).
 static inline int red_grid(int64_t n) {
-  const int64_t g = (n + 8 * RED_THREADS - 1) / (8 * RED_THREADS);
+  const int64_t g2 = std::min<int64_t>((n + 2 * RED_THREADS - 1) / (2 * RED_THREADS), 304);
+  const int64_t g = std::max<int64_t>(g2, (n + 8 * RED_THREADS - 1) / (8 * RED_THREADS));
   return (int)(g < 1 ? 1 : (g > RED_BLOCKS ? RED_BLOCKS : g));
 }
 static inline unsigned* red_counters(double* scratch) { return reinterpret_cast<unsigned*>(scratch + (size_t)RED_BLOCKS * 64); }
