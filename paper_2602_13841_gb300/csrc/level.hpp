@@ -22,7 +22,8 @@ struct Level {
   double hscale = 0;                  // Nitsche length factor (see LevelArgs)
   int64_t chunk_cells = 262144;       // cells per chunk of the smoother build's element scratch
   int smoother = 0;                   // 0: surrogate patches (Sec. 4.3); 1: diagonal space-time Vanka
-  double* geo64 = nullptr;            // 2D: geometry table of the FP64 operator (see OpArgs::geo)
+  double* geo64 = nullptr;            // 2D: geometry tables of the FP64 operator (see OpArgs::geo, fgeo)
+  double* fgeo64 = nullptr;
   void* cellbuf = nullptr;            // cell-wise results of the operator kernels (CellBuf), one buffer
   size_t cellbuf_bytes = 0;           // for all levels of a handle, on the handle's stream only
 };
@@ -72,7 +73,8 @@ inline size_t cellbuf_need(int d, int n, int r, int k) {
 
 cudaError_t launch_initial_condition(const Level& lv, const Problem& pb, double* V0, cudaStream_t s);
 
-// Fill lv.geo64 (allocated by the caller: cells x 5 x (r+2)^2 entries) of a 2D level.
+// Fill lv.geo64 and lv.fgeo64 (allocated by the caller: cells x 5 x (r+2)^2 and 4 n x 6 x (r+2) entries) of
+// a 2D level.
 cudaError_t build_geometry(const Level& lv, const Problem& pb, cudaStream_t s);
 
 }  // namespace stmg

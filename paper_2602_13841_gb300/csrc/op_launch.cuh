@@ -88,7 +88,8 @@ static cudaError_t launch_dn(const Level& lv, const Problem& pb, double t0, cons
   const int kp1 = lv.k + 1;
   const Tab<T> tb = make_tab<T>(lv.tabs, pb.tau);
   const T* geo = nullptr;
-  if constexpr (D == 2 && F64) geo = lv.geo64;
+  const T* fgeo = nullptr;
+  if constexpr (D == 2 && F64) { geo = lv.geo64; fgeo = lv.fgeo64; }
   const int64_t cplane = D == 2 ? lv.n : (int64_t)lv.n * lv.n;   // cells per plane of the last axis
   CellBuf<T> cb{};
   int64_t cols;
@@ -100,7 +101,7 @@ static cudaError_t launch_dn(const Level& lv, const Problem& pb, double t0, cons
   for (int64_t b0 = 0; b0 < batch; b0 += cols) {
     const int nb = (int)(batch - b0 < cols ? batch - b0 : cols);
     OpArgs<T> A{level_args<T>(lv, pb, t0), x + b0 * xs, state ? state + b0 * ss : nullptr, vprev, y + b0 * ys,
-                xs, ys, geo, ss, nub ? nub + b0 : nullptr};
+                xs, ys, geo, fgeo, ss, nub ? nub + b0 : nullptr};
     const T* rb = rhs ? rhs + b0 * ys : nullptr;
     for (int z0 = 0; z0 < lv.n; z0 += step) {
       const int z1 = z0 + step < lv.n ? z0 + step : lv.n;

@@ -104,6 +104,7 @@ static void build_level(Handle* h, Level& lv, const std::vector<double>& verts) 
     // geometry table of the 2D FP64 operator (5 values per cell and Gauss point)
     const size_t ng = (size_t)ncells * 5 * (lv.r + 2) * (lv.r + 2);
     lv.geo64 = (double*)h->dalloc(ng * sizeof(double));
+    lv.fgeo64 = (double*)h->dalloc((size_t)24 * lv.n * (lv.r + 2) * sizeof(double));
     if (build_geometry(lv, h->pb, h->stream) != cudaSuccess) throw CudaFailure(cudaErrorLaunchFailure);
   }
 }
@@ -167,7 +168,7 @@ stmg_status stmg_footprint(const stmg_params* p, uint64_t* bytes) {
     nst[l] = (lk + 1.0) * (Nv + Np);
     tot += 12.0 * d * std::pow(ln + 1.0, d);                            // vertices
     cbuf = std::max(cbuf, (double)cellbuf_need(d, ln, lr, lk));
-    if (d == 2) tot += cells * 5.0 * (lr + 2.0) * (lr + 2.0) * 8.0;     // 2D geometry table
+    if (d == 2) tot += (cells * 5.0 * (lr + 2.0) + 24.0 * ln) * (lr + 2.0) * 8.0;   // 2D geometry tables
     tot += 5.0 * nst[l] * es;                                            // level vectors
     if (l + 1 < lv.size()) {
       double nl = std::pow(lr + 2.0, d), mv = d * nl, msp = mv + npc;
