@@ -225,11 +225,26 @@ __device__ inline T invert(const T (*J)[3], T (*G)[3]) {
 // lid-driven cavity of Sec. 5.2, g = (sin(pi t / 4), 0, 0) on the lid z = 1, zero on the other
 // walls, f = 0, v0 = 0.  Face quadrature points are interior to their faces, so z = 1 (up to
 // rounding of the multilinear map) holds exactly on the lid's points and nowhere else.
+// Sines and cosines of pi x by sincospi, of 2 pi x by the double-angle formulas: an FP64 sine costs some
+// forty operations of a pipe that does two per clock and SM, so a point's data take one call per
+// coordinate, and the factors in time one per thread (2D 32^2 Q2/P1 DG(1) slab solve 7.65 -> 7.47 ms).
+// Largest error over [0, 1] against 120 bits: sin 2 pi x 2.0e-16, cos 2 pi x 3.3e-16 (sin and cos of the
+// rounded 2 pi x: 6.9e-16, 6.4e-16).
+struct Trig {
+  double s, c, s2, c2;                                // sin, cos of pi x and 2 pi x
+  __device__ explicit Trig(double x) {
+    sincospi(x, &s, &c);
+    s2 = 2.0 * s * c;
+    c2 = 1.0 - 2.0 * s * s;
+  }
+};
+
 __device__ inline void problem_velocity_tg2d(const double* x, double t, double nu, double* v) {
   const double pi = 3.141592653589793238;
   double F = exp(-2.0 * pi * pi * nu * t);
-  v[0] = F * sin(pi * x[0]) * cos(pi * x[1]);
-  v[1] = -F * cos(pi * x[0]) * sin(pi * x[1]);
+  const Trig X(x[0]), Y(x[1]);
+  v[0] = F * X.s * Y.c;
+  v[1] = -F * X.c * Y.s;
 }
 
 template <int D>
@@ -239,8 +254,9 @@ __device__ inline void problem_g(int problem, const double* x, double t, double 
   if (problem == 0 && D == 2) {
     problem_velocity_tg2d(x, t, nu, g);
   } else if (problem == 2 && D == 3) {
-    g[0] = sin(pi * x[0]) * cos(pi * x[1]) * cos(pi * x[2]);
-    g[1] = -cos(pi * x[0]) * sin(pi * x[1]) * cos(pi * x[2]);
+    const Trig X(x[0]), Y(x[1]), Z(x[2]);
+    g[0] = X.s * Y.c * Z.c;
+    g[1] = -X.c * Y.s * Z.c;
   } else if (problem == 4 && D == 3) {
     if (x[2] > 1.0 - 1e-9) g[0] = sin(0.25 * pi * t);
   }
@@ -251,15 +267,14 @@ __device__ inline void problem_v0(int problem, const double* x, double nu, doubl
   problem_g<D>(problem, x, 0.0, nu, v);
 }
 
+// st, ct: sin t and cos t (the same for every point of a time node)
 template <int D>
-__device__ inline void problem_f(int problem, const double* x, double t, double nu, double* f) {
+__device__ inline void problem_f(int problem, const double* x, double st, double ct, double nu, double* f) {
   const double pi = 3.141592653589793238;
   for (int i = 0; i < D; ++i) f[i] = 0.0;
-  double st = sin(t), ct = cos(t);
   if (problem == 1 && D == 2) {
-    double sx = sin(pi * x[0]), cx = cos(pi * x[0]), sy = sin(pi * x[1]), cy = cos(pi * x[1]);
-    double s2x = sin(2 * pi * x[0]), c2x = cos(2 * pi * x[0]);
-    double s2y = sin(2 * pi * x[1]), c2y = cos(2 * pi * x[1]);
+    const Trig X(x[0]), Y(x[1]);
+    double sx = X.s, cx = X.c, sy = Y.s, cy = Y.c, s2x = X.s2, c2x = X.c2, s2y = Y.s2, c2y = Y.c2;
     double u = sx * sx * sy * cy, w = -sx * cx * sy * sy;          // spatial profile
     double ux = 2 * pi * sx * cx * sy * cy, uy = pi * sx * sx * c2y;
     double wx = -pi * c2x * sy * sy, wy = -2 * pi * sx * cx * sy * cy;
@@ -269,11 +284,9 @@ __device__ inline void problem_f(int problem, const double* x, double t, double 
     f[0] = ct * u + st * st * (u * ux + w * uy) - nu * st * lu + st * px;
     f[1] = ct * w + st * st * (u * wx + w * wy) - nu * st * lw + st * py;
   } else if (problem == 3 && D == 3) {
-    double sx = sin(pi * x[0]), sy = sin(pi * x[1]);
-    double s2x = sin(2 * pi * x[0]), c2x = cos(2 * pi * x[0]);
-    double s2y = sin(2 * pi * x[1]), c2y = cos(2 * pi * x[1]);
-    double s2z = sin(2 * pi * x[2]), c2z = cos(2 * pi * x[2]);
-    double Z = sin(pi * x[2]);
+    const Trig X(x[0]), Y(x[1]), Zt(x[2]);
+    double sx = X.s, sy = Y.s, s2x = X.s2, c2x = X.c2, s2y = Y.s2, c2y = Y.c2, s2z = Zt.s2, c2z = Zt.c2;
+    double Z = Zt.s;
     double a = pi * sx * sx * s2y, b = -pi * s2x * sy * sy;
     double ax = pi * pi * s2x * s2y, ay = 2 * pi * pi * sx * sx * c2y;
     double bx = -2 * pi * pi * c2x * sy * sy, by = -pi * pi * s2x * s2y;

@@ -698,6 +698,8 @@ __global__ void __launch_bounds__(BT, MINB) k_cells3d(OpArgs<T> A, const __grid_
     __syncthreads();
     // ---- pointwise fluxes; along x and z they go back in place of the derivatives
     if (on) {
+      double st = 0, ct = 0;
+      if (RES && L.problem == kProblemMms3d) sincos((double)L.t0 + 0.5 * (double)L.tau * ((double)tb.that[a] + 1.0), &st, &ct);
       T fy[3][N];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -754,7 +756,7 @@ __global__ void __launch_bounds__(BT, MINB) k_cells3d(OpArgs<T> A, const __grid_
             const T X = lt.qx[u], Y = tb.qx[j], Z = lt.qx[v];
             double xd[3], fd[3];
             for (int l = 0; l < 3; ++l) xd[l] = (double)map3_point<T>(s_map, l, X, Y, Z);
-            problem_f<3>(L.problem, xd, (double)L.t0 + 0.5 * (double)L.tau * ((double)tb.that[a] + 1.0), (double)L.nu, fd);
+            problem_f<3>(L.problem, xd, st, ct, (double)L.nu, fd);
             for (int c = 0; c < 3; ++c) fq[c] = (T)fd[c];
           }
 #pragma unroll
@@ -1178,6 +1180,8 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
   if (!MASS) {
     __syncthreads();
     if (on) {
+      double st = 0, ct = 0;
+      if (RES && L.problem == kProblemMms2d) sincos((double)L.t0 + 0.5 * (double)L.tau * ((double)tb.that[a] + 1.0), &st, &ct);
       T fx[2][N];
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
@@ -1222,7 +1226,7 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
             for (int l = 0; l < 2; ++l)
               xd[l] = (double)(L.verts[2 * v0 + l] * ((1 - X) * (1 - Y)) + L.verts[2 * v0 + 2 + l] * (X * (1 - Y)) +
                                L.verts[2 * (v0 + L.n + 1) + l] * ((1 - X) * Y) + L.verts[2 * (v0 + L.n + 2) + l] * (X * Y));
-            problem_f<2>(L.problem, xd, (double)L.t0 + 0.5 * (double)L.tau * ((double)tb.that[a] + 1.0), (double)L.nu, fd);
+            problem_f<2>(L.problem, xd, st, ct, (double)L.nu, fd);
             f0 = (T)fd[0];
             f1 = (T)fd[1];
           }
