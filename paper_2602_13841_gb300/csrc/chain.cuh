@@ -1,0 +1,40 @@
+// Chained launches (programmatic dependent launch).  A V-cycle and an FGMRES iteration are hundreds of
+// kernels of a few microseconds, each reading what the one before wrote, so the time between two of
+// them counts.  A chained kernel may be scheduled while its predecessor's last blocks run: its first
+// statement, chain_begin(), waits until that grid has ended and its writes are visible, then lets the
+// next one be scheduled.  Nothing is read or written before it, so every order of a plain launch holds: a
+// grid ends only after its own wait, hence after all grids before it.  A predecessor without
+// chain_begin(), a copy, a memset or an event wait is ordered as by a plain launch; a chained launch
+// captures into a graph like a plain one.  Inputs that earlier kernels of the chain write are not
+// declared const __restrict__: the loads of such pointers may be moved above the wait.
+// Plain -> chained: 2D 8^2 Q2/P1 DG(1) FP64 apply 30.7 -> 27.1 us, 2D 256^2 Q3/P2 DG(2) FP32 apply 57.3 ->
+// 52.8, 2D 32^2 Q2/P1 DG(1) slab solve 7.52 -> 6.71 ms.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <utility>
+
+namespace stmg {
+
+__device__ __forceinline__ void chain_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launch a kernel that opens with chain_begin(), CHAINED or plainly.  An error is left for cudaGetLastError.
+template <bool CHAINED = true, typename... P, typename... A>
+static void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = CHAINED ? 1 : 0;
+  cudaLaunchKernelEx(&c, kern, std::forward<A>(args)...);
+}
+
+}  // namespace stmg

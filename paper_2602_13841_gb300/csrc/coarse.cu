@@ -5,6 +5,7 @@
 // with one step of iterative refinement against the bordered matrix.
 #include "mg.hpp"
 #include "op_launch.cuh"
+#include "chain.cuh"
 #include "counters.hpp"
 
 namespace stmg {
@@ -282,9 +283,10 @@ cudaError_t coarse_invert(const double* A, double* Ainv, double* work, double* p
 // its 32 groups of 8 threads every 32nd column; their sums meet in shared memory in a fixed order.
 // FP64 on few SMs is slow, so small systems are spread over n / 8 blocks (n = 126: 10.2 -> 3.7 us).
 template <typename T, int STEP>
-__global__ void __launch_bounds__(256) k_coarse_mv(const double* __restrict__ A, int n, int nc, const T* __restrict__ b,
-                                                   const double* __restrict__ x1, const double* __restrict__ r,
+__global__ void __launch_bounds__(256) k_coarse_mv(const double* A, int n, int nc, const T* b, const double* x1,
+                                                   const double* r,
                                                    double* __restrict__ y, T* __restrict__ out) {
+  chain_begin();
   __shared__ double part[32][9];
   A += (int64_t)blockIdx.y * n * n;                   // blockIdx.y: independent slot
   b += (int64_t)blockIdx.y * nc;
@@ -324,9 +326,9 @@ template <typename T>
 cudaError_t coarse_apply(const double* Ainv, const double* A, int n, int nc, const T* b, T* out, double* x1, double* r,
                          cudaStream_t s, int slots) {
   const dim3 grid((n + 7) / 8, slots);
-  k_coarse_mv<T, 0><<<grid, 256, 0, s>>>(Ainv, n, nc, b, nullptr, nullptr, x1, nullptr);
-  k_coarse_mv<T, 1><<<grid, 256, 0, s>>>(A, n, nc, b, x1, nullptr, r, nullptr);
-  k_coarse_mv<T, 2><<<grid, 256, 0, s>>>(Ainv, n, nc, b, x1, r, nullptr, out);
+  launch_chained(k_coarse_mv<T, 0>, grid, 256, 0, s, Ainv, n, nc, b, nullptr, nullptr, x1, nullptr);
+  launch_chained(k_coarse_mv<T, 1>, grid, 256, 0, s, A, n, nc, b, x1, nullptr, r, nullptr);
+  launch_chained(k_coarse_mv<T, 2>, grid, 256, 0, s, Ainv, n, nc, b, x1, r, nullptr, out);
   note_launch(3);
   return cudaGetLastError();
 }

@@ -39,6 +39,7 @@
 #pragma once
 #include <type_traits>
 
+#include "chain.cuh"
 #include "common.cuh"
 
 namespace stmg {
@@ -496,7 +497,8 @@ __device__ __forceinline__ void face3d(const OpArgs<T>& A, const Tab<T>& tb, con
 
 template <typename T, int N, int MODE, int BT, int MINB>
 __global__ void __launch_bounds__(BT, MINB) k_cells3d(OpArgs<T> A, const __grid_constant__ Tab<T> tb, CellBuf<T> cb,
-                                                      int64_t c0, int64_t c1, int cpb, const T* __restrict__ rhs) {
+                                                      int64_t c0, int64_t c1, int cpb, const T* rhs) {
+  chain_begin();
   constexpr bool RES = MODE == MR, MASS = MODE == MM, JAC = MODE == MJ;
   constexpr int NN = N * N, Q = N * NN, PL = plane3<N>(), QP = arr3<N>(), NPC = npress<3, N>();
   constexpr int GS = group3<N>();
@@ -1036,7 +1038,8 @@ __device__ __forceinline__ void face2d(const OpArgs<T>& A, const Tab<T>& tb, con
 
 template <typename T, int N, int MODE, int BT, int MINB>
 __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_constant__ Tab<T> tb, CellBuf<T> cb,
-                                                      int64_t c0, int64_t c1, int cpb, const T* __restrict__ rhs) {
+                                                      int64_t c0, int64_t c1, int cpb, const T* rhs) {
+  chain_begin();
   constexpr bool RES = MODE == MR, MASS = MODE == MM, JAC = MODE == MJ;
   constexpr int Q = N * N, NPC = npress<2, N>();
   constexpr int GS = group2<N>();
@@ -1342,6 +1345,7 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
 template <typename T, int D, int N, int KP1>
 __global__ void k_node_sum(CellBuf<T> cb, const T* src, T* y, T alpha, int n, int N1, int64_t nnodes, int64_t Nv,
                            int64_t ys, int g0, int64_t count, const int* skip) {
+  chain_begin();
   if (skip && *skip) return;
   y += blockIdx.y * ys;
   if (src) src += blockIdx.y * ys;

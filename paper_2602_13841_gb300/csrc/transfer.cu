@@ -5,6 +5,7 @@
 
 #include "handle.hpp"
 #include "transfer.hpp"
+#include "chain.cuh"
 #include "counters.hpp"
 
 namespace stmg {
@@ -151,6 +152,7 @@ struct TransferArgs {
 
 template <typename T, int D>
 __global__ void k_transfer(const __grid_constant__ TransferArgs<T> A) {
+  chain_begin();
   const T* in = A.in + blockIdx.y * A.zin;            // blockIdx.y: independent slot
   T* out = A.out + blockIdx.y * A.zout;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -259,8 +261,8 @@ static cudaError_t transfer_launch(const Transfer& tr, const Line1D& op, const L
   A.PT = ptab<T>(tr);
   A.pin = li.Np; A.pout = lo.Np; A.zin = li.Nst; A.zout = lo.Nst;
   const dim3 grid((unsigned)((A.total + 127) / 128), (unsigned)slots);
-  if (li.d == 2) k_transfer<T, 2><<<grid, 128, 0, s>>>(A);
-  else k_transfer<T, 3><<<grid, 128, 0, s>>>(A);
+  if (li.d == 2) launch_chained(k_transfer<T, 2>, grid, 128, 0, s, A);
+  else launch_chained(k_transfer<T, 3>, grid, 128, 0, s, A);
   note_launch();
   return cudaGetLastError();
 }

@@ -53,6 +53,8 @@ struct StreamShape {
 // A batch of U chunks of a thread: 16 bytes each of a complex block, 8 of a real one.
 template <bool C, int U> struct ChunkBatch { uint32_t w[U][C ? 4 : 2]; };
 
+// The inverses are written by kernels that end before this one starts (they are not chained), so they may
+// take the non-coherent path; volatile keeps the loads after chain_begin().
 // q: the thread's chunk of the batch's first column; STEP bytes between its columns; `left` columns from
 // the first one on exist (chunks past them are zero).
 template <bool C, int U, int STEP>
@@ -62,10 +64,10 @@ __device__ __forceinline__ void load_batch(ChunkBatch<C, U>& c, const unsigned c
   for (int u = 0; u < U; ++u) {
     if (u * js_step < left) {
       if constexpr (C)
-        asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
+        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
             : "=r"(c.w[u][0]), "=r"(c.w[u][1]), "=r"(c.w[u][2]), "=r"(c.w[u][3]) : "l"(q + u * STEP), "l"(pol));
       else
-        asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
+        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
             : "=r"(c.w[u][0]), "=r"(c.w[u][1]) : "l"(q + u * STEP), "l"(pol));
     } else {
 #pragma unroll
@@ -119,9 +121,10 @@ __device__ __forceinline__ void use_batch(const ChunkBatch<C, U>& c, const T* r,
 // first; smaller levels are read again by the next sweep and stay.
 template <typename T, typename SI, int D, int N, int KP1>
 __global__ void __launch_bounds__(StreamShape<T, SI, D, N>::THREADS, StreamShape<T, SI, D, N>::BLOCKS)
-k_vanka_stream(LevelArgs<T> L, const SI* __restrict__ inv, const float* __restrict__ scale, const T* __restrict__ res,
+k_vanka_stream(LevelArgs<T> L, const SI* inv, const float* scale, const T* res,
                T* __restrict__ d, T omega_p, const __grid_constant__ TEig<T> te, CellBuf<T> cb, int64_t c0,
                SlotStrides zs, int first, int stream) {
+  chain_begin();
   using Sh = StreamShape<T, SI, D, N>;
   constexpr int MS = Sh::MS, MV = Sh::MV, ST = Sh::ST, RC = Sh::RC, P = Sh::P, JS = Sh::JS, U = Sh::U, NB = Sh::NB;
   constexpr int NL = Shape<D, N>::Q, NPC = MS - MV, NT = Sh::THREADS, MP = Sh::MP, ROWS = (MS + NT - 1) / NT;

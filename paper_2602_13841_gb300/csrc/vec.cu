@@ -2,6 +2,7 @@
 // reductions in a fixed order (block partial sums, then one block per result).
 #include <algorithm>
 #include "vec.cuh"
+#include "chain.cuh"
 #include "counters.hpp"
 
 namespace stmg {
@@ -14,27 +15,29 @@ static inline int grid_for(int64_t n) {
 }
 
 template <typename T>
-__global__ void k_axpby(int64_t n, T a, const T* __restrict__ x, T b, T* __restrict__ y) {
+__global__ void k_axpby(int64_t n, T a, const T* x, T b, T* __restrict__ y) {
+  chain_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = a * x[i] + b * y[i];
 }
 
 template <typename T>
 cudaError_t vaxpby(int64_t n, T a, const T* x, T b, T* y, cudaStream_t s) {
-  k_axpby<T><<<grid_for(n), 256, 0, s>>>(n, a, x, b, y);
+  launch_chained(k_axpby<T>, grid_for(n), 256, 0, s, n, a, x, b, y);
   note_launch();
   return cudaGetLastError();
 }
 
 template <typename S, typename T>
-__global__ void k_copy(int64_t n, const S* __restrict__ x, T* __restrict__ y) {
+__global__ void k_copy(int64_t n, const S* x, T* __restrict__ y) {
+  chain_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = (T)x[i];
 }
 
 template <typename S, typename T>
 cudaError_t vcopy(int64_t n, const S* x, T* y, cudaStream_t s) {
-  k_copy<S, T><<<grid_for(n), 256, 0, s>>>(n, x, y);
+  launch_chained(k_copy<S, T>, grid_for(n), 256, 0, s, n, x, y);
   note_launch();
   return cudaGetLastError();
 }
@@ -84,8 +87,9 @@ __device__ __forceinline__ bool last_block(unsigned* count) {
 }
 
 template <typename T>
-__global__ void k_dots(int64_t n, int m, const T* __restrict__ X, int64_t ldx, const T* __restrict__ w, double* part,
+__global__ void k_dots(int64_t n, int m, const T* X, int64_t ldx, const T* w, double* part,
                        double* __restrict__ out, unsigned* count) {
+  chain_begin();
   __shared__ double red[DOTS_PER_ROW][RED_THREADS];
   const int l0 = blockIdx.y * DOTS_PER_ROW;
   const int cnt = m - l0 < DOTS_PER_ROW ? m - l0 : DOTS_PER_ROW;
@@ -132,16 +136,16 @@ cudaError_t vdots(int64_t n, int m, const T* X, int64_t ldx, const T* w, double*
                   cudaStream_t s) {
   if (m <= 0) return cudaSuccess;
   if (m > 64) return cudaErrorInvalidValue;
-  k_dots<T><<<dim3(red_grid(n), (m + DOTS_PER_ROW - 1) / DOTS_PER_ROW), RED_THREADS, 0, s>>>(
-      n, m, X, ldx, w, scratch, out, red_counters(scratch));
+  launch_chained(k_dots<T>, dim3(red_grid(n), (m + DOTS_PER_ROW - 1) / DOTS_PER_ROW), RED_THREADS, 0, s, n, m, X, ldx, w, scratch, out, red_counters(scratch));
   note_launch();
   return cudaGetLastError();
 }
 
 // w -= sum_l h[l] X[l]; NORM: also out = sum_i w_i^2 of the result (the same two-stage sum).
 template <typename T, bool NORM>
-__global__ void k_sub_comb(int64_t n, int m, const T* __restrict__ X, int64_t ldx, const double* __restrict__ h,
+__global__ void k_sub_comb(int64_t n, int m, const T* X, int64_t ldx, const double* h,
                            T* __restrict__ w, double* part, double* __restrict__ out, unsigned* count) {
+  chain_begin();
   __shared__ double hs[64];
   __shared__ double red[1][RED_THREADS];
   if (threadIdx.x < m) hs[threadIdx.x] = h[threadIdx.x];
@@ -172,7 +176,7 @@ template <typename T>
 cudaError_t vsub_comb(int64_t n, int m, const T* X, int64_t ldx, const double* h, T* w, cudaStream_t s) {
   if (m <= 0) return cudaSuccess;
   if (m > 64) return cudaErrorInvalidValue;
-  k_sub_comb<T, false><<<grid_for(n), RED_THREADS, 0, s>>>(n, m, X, ldx, h, w, nullptr, nullptr, nullptr);
+  launch_chained(k_sub_comb<T, false>, grid_for(n), RED_THREADS, 0, s, n, m, X, ldx, h, w, (double*)nullptr, (double*)nullptr, (unsigned*)nullptr);
   note_launch();
   return cudaGetLastError();
 }
@@ -181,15 +185,16 @@ template <typename T>
 cudaError_t vsub_comb_norm(int64_t n, int m, const T* X, int64_t ldx, const double* h, T* w, double* out, double* scratch,
                            cudaStream_t s) {
   if (m <= 0 || m > 64) return cudaErrorInvalidValue;
-  k_sub_comb<T, true><<<red_grid(n), RED_THREADS, 0, s>>>(n, m, X, ldx, h, w, scratch, out, red_counters(scratch));
+  launch_chained(k_sub_comb<T, true>, red_grid(n), RED_THREADS, 0, s, n, m, X, ldx, h, w, scratch, out, red_counters(scratch));
   note_launch();
   return cudaGetLastError();
 }
 
 struct Coef64 { double v[64]; };
 
-__global__ void k_add_comb(int64_t n, int m, const double* __restrict__ Z, int64_t ldz, Coef64 y,
+__global__ void k_add_comb(int64_t n, int m, const double* Z, int64_t ldz, Coef64 y,
                            double* __restrict__ x) {
+  chain_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     double acc = x[i];
     for (int l = 0; l < m; ++l) acc += y.v[l] * Z[l * ldz + i];
@@ -203,13 +208,14 @@ cudaError_t vadd_comb_host(int64_t n, int m, const double* Z, int64_t ldz, const
   if (m > 64) return cudaErrorInvalidValue;
   Coef64 c{};
   for (int l = 0; l < m; ++l) c.v[l] = y[l];
-  k_add_comb<<<grid_for(n), 256, 0, s>>>(n, m, Z, ldz, c, x);
+  launch_chained(k_add_comb, grid_for(n), 256, 0, s, n, m, Z, ldz, c, x);
   note_launch();
   return cudaGetLastError();
 }
 
 template <typename T>
-__global__ void k_scale_inv_dev(int64_t n, const T* __restrict__ x, const double* __restrict__ nrm, T* __restrict__ y) {
+__global__ void k_scale_inv_dev(int64_t n, const T* x, const double* nrm, T* __restrict__ y) {
+  chain_begin();
   const double f = 1.0 / *nrm;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = (T)((double)x[i] * f);
@@ -217,20 +223,21 @@ __global__ void k_scale_inv_dev(int64_t n, const T* __restrict__ x, const double
 
 template <typename T>
 cudaError_t vscale_inv_dev(int64_t n, const T* x, const double* nrm, T* y, cudaStream_t s) {
-  k_scale_inv_dev<T><<<grid_for(n), 256, 0, s>>>(n, x, nrm, y);
+  launch_chained(k_scale_inv_dev<T>, grid_for(n), 256, 0, s, n, x, nrm, y);
   note_launch();
   return cudaGetLastError();
 }
 
 template <typename T>
-__global__ void k_scale(int64_t n, T a, const T* __restrict__ x, T* __restrict__ y) {
+__global__ void k_scale(int64_t n, T a, const T* x, T* __restrict__ y) {
+  chain_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = a * x[i];
 }
 
 template <typename T>
 cudaError_t vscale(int64_t n, T a, const T* x, T* y, cudaStream_t s) {
-  k_scale<T><<<grid_for(n), 256, 0, s>>>(n, a, x, y);
+  launch_chained(k_scale<T>, grid_for(n), 256, 0, s, n, a, x, y);
   note_launch();
   return cudaGetLastError();
 }
@@ -247,13 +254,14 @@ cudaError_t vfill(int64_t n, T v, T* x, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-__global__ void k_finite(int64_t n, const double* __restrict__ x, int* flag) {
+__global__ void k_finite(int64_t n, const double* x, int* flag) {
+  chain_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     if (!isfinite(x[i])) *flag = 1;
 }
 
 cudaError_t vfinite(int64_t n, const double* x, int* flag, cudaStream_t s) {
-  k_finite<<<grid_for(n), 256, 0, s>>>(n, x, flag);
+  launch_chained(k_finite, grid_for(n), 256, 0, s, n, x, flag);
   note_launch();
   return cudaGetLastError();
 }
