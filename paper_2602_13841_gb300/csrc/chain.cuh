@@ -21,9 +21,10 @@ __device__ __forceinline__ void chain_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Launch a kernel that opens with chain_begin(), CHAINED or plainly.  An error is left for cudaGetLastError.
-template <bool CHAINED = true, typename... P, typename... A>
-static void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+// Launch a kernel that opens with chain_begin(), chained or plainly.  An error is left for cudaGetLastError.
+template <typename... P, typename... A>
+static void launch_if_chained(bool chained, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                              A&&... args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
@@ -33,8 +34,13 @@ static void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t sme
   c.dynamicSmemBytes = smem;
   c.stream = s;
   c.attrs = &at;
-  c.numAttrs = CHAINED ? 1 : 0;
+  c.numAttrs = chained ? 1 : 0;
   cudaLaunchKernelEx(&c, kern, std::forward<A>(args)...);
+}
+
+template <typename... P, typename... A>
+static void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  launch_if_chained(true, kern, grid, block, smem, s, std::forward<A>(args)...);
 }
 
 }  // namespace stmg

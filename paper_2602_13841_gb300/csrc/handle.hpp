@@ -15,7 +15,7 @@
 namespace stmg {
 
 // Kernel classes of the profile: FP64 Jacobian apply, preconditioner-precision Jacobian apply,
-// residual, Vanka patch apply (one launch per colour), Vanka build, mass apply.
+// residual, Vanka patch apply (one span per sweep), Vanka build, mass apply.
 enum KernelClass { KC_APPLY64 = 0, KC_APPLYP = 1, KC_RESIDUAL = 2, KC_VANKA_APPLY = 3, KC_VANKA_BUILD = 4,
                    KC_MASS = 5, KC_VANKA_APPLY0 = 6, KC_COUNT = 7 };
 

@@ -58,21 +58,28 @@ static bool plan_cellbuf(const Level& lv, int batch, CellBuf<T>& cb, int64_t& co
   return true;
 }
 
-// Whether an operator's launches are chained: all but 3D FP64, whose cell kernels run in a few long waves.
-// Placed while the previous grid still holds room, their blocks spread unevenly over the SMs: 16^3 Q3/P2
-// DG(2) residual 743-745 us with both launches or the cells alone chained, 731 with the node sums alone, 727
-// with neither.
-template <typename T, int D> constexpr bool chained_cells() { return !(D == 3 && sizeof(T) == 8); }
+// Whether an operator's two launches are chained, by the blocks of its cell kernel.  Blocks placed while the
+// previous grid still holds room spread unevenly over the SMs, which costs a grid of about one wave more
+// than the gap it saves; grids of up to a block or two per SM and those of many waves gain (2D, in a graph,
+// chained / plain: FP32 Q2/P1 DG(0) 32^2 7.1 / 7.7 us, 192^2 11.4 / 10.1; Q3/P2 DG(0) 128^2 11.6 / 10.3; Q3/P2
+// DG(2) 96^2 13.9 / 12.7, 256^2 50.6 / 51.0; FP64 Q2/P1 DG(1) 8^2 26.2 / 26.7, 64^2 39.2 / 36.1; Q3/P2 DG(2) 32^2
+// 49.0 / 39.7, 256^2 865 / 866).  3D FP64: few long waves, 16^3 Q3/P2 DG(2) residual 745 / 727 us.
+template <typename T, int D>
+static bool chained_cells(int64_t blocks) {
+  constexpr int64_t sms = 152;
+  if (sizeof(T) == 8) return D == 2 && blocks <= sms;
+  return blocks <= 2 * sms || blocks >= 20 * sms;
+}
 
 // Node sums of the cell planes z0 .. z1 - 1 (see k_node_sum).
 template <typename T, int D, int N>
 static void launch_node_sum(const Level& lv, const CellBuf<T>& cb, const T* src, T* y, T alpha, int64_t ys, int z0,
-                            int z1, int columns, const int* skip, cudaStream_t s) {
+                            int z1, int columns, const int* skip, cudaStream_t s, bool chained = true) {
   const int g0 = z0 * (N - 1), g1 = z1 == lv.n ? lv.N1 : z1 * (N - 1);
   const int64_t nodes = (int64_t)(g1 - g0) * (D == 2 ? (int64_t)lv.N1 : (int64_t)lv.N1 * lv.N1);
   const int64_t blocks = (nodes + 127) / 128;
   auto kern = lv.k == 0 ? k_node_sum<T, D, N, 1> : lv.k == 1 ? k_node_sum<T, D, N, 2> : k_node_sum<T, D, N, 3>;
-  launch_chained<chained_cells<T, D>()>(kern, dim3((unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), columns), 128, 0, s,
+  launch_if_chained(chained, kern, dim3((unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), columns), 128, 0, s,
                  cb, src, y, alpha, lv.n, lv.N1, lv.nnodes, lv.Nv, ys, g0, nodes, skip);
   note_launch();
 }
@@ -91,7 +98,6 @@ static cudaError_t launch_dn(const Level& lv, const Problem& pb, double t0, cons
   // FP64 at 64^3 Q2/P1 DG(2) 192 x 2 12.6 ms, 128 x 3 14.0 (more lanes idle)
   constexpr int BT = D == 2 ? 128 : (N == 5 ? 256 : (F64 ? 192 : 128));
   constexpr int MINB = D == 2 ? (F64 ? 4 : 7) : (N == 5 ? (F64 ? 1 : 2) : (F64 ? 2 : 4));
-  constexpr bool CHAINED = chained_cells<T, D>();
   const int kp1 = lv.k + 1;
   const Tab<T> tb = make_tab<T>(lv.tabs, pb.tau);
   const T* geo = nullptr;
@@ -120,10 +126,12 @@ static cudaError_t launch_dn(const Level& lv, const Problem& pb, double t0, cons
         if (e != cudaSuccess) return e;
       }
       const int threads = (cpb * kp1 * TPG + 31) / 32 * 32;
-      launch_chained<CHAINED>(kern, dim3((unsigned)((c1 - c0 + cpb - 1) / cpb), nb), threads, smem, stream, A, tb,
+      const int64_t blocks = (c1 - c0 + cpb - 1) / cpb;
+      const bool chained = chained_cells<T, D>(blocks * nb);
+      launch_if_chained(chained, kern, dim3((unsigned)blocks, nb), threads, smem, stream, A, tb,
                      cb, c0, c1, cpb, rb);
       note_launch();
-      launch_node_sum<T, D, N>(lv, cb, rb, A.y, rhs ? (T)-1 : (T)1, ys, z0, z1, nb, nullptr, stream);
+      launch_node_sum<T, D, N>(lv, cb, rb, A.y, rhs ? (T)-1 : (T)1, ys, z0, z1, nb, nullptr, stream, chained);
     }
   }
   return cudaGetLastError();

@@ -14,8 +14,9 @@
 //      M^tau = diag(w_a).  S~_K is inverted through its time diagonalisation, one spatial system per
 //      eigenvalue, by Gauss-Jordan elimination with partial pivoting (vanka_patch.cuh); the inverse is
 //      stored column-major per cell.
-// Sweep (additive, damped): d <- d + omega sum_K R_K^T S~_K^{-1} R_K (rhs - J d); cells are
-// updated in 2^d colours so that the scatter is race free and deterministic.
+// Sweep (additive, damped): d <- d + omega sum_K R_K^T S~_K^{-1} R_K (rhs - J d); the cells' corrections
+// are added per node in a fixed order (vanka_stream.cuh; the other smoothers: cells in 2^d colours), so
+// that the scatter is race free and deterministic.
 #pragma once
 #include <cuda_fp16.h>
 

@@ -103,7 +103,7 @@ __host__ __device__ inline size_t apply_exact_smem(int mst, int ms, size_t t) {
 
 // d[patch] += W~ S_K^{-1} res[patch] for the cells of one colour; one block per cell, thread i owns
 // patch row i (time node i / m_s, spatial DoF i % m_s).  The inverse is staged by bulk copies on an
-// mbarrier with the bounded wait of k_vanka_apply.
+// mbarrier with a bounded wait (mbar_wait_bounded).
 template <typename T, int D, int N>
 __global__ void k_vanka_apply_exact(LevelArgs<T> L, const T* __restrict__ inv, const T* __restrict__ res,
                                     T* __restrict__ d, T omega, T omega_p, int kp1, int npc, ColorInfo ci,
