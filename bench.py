@@ -576,7 +576,7 @@ def main():
 
 
 def operator_apply(S, U, stream, dev, w, args, peaks, reps=25, warm=5):
-    """Finest-level y = J(U) x (zeroing of y and every colour launch), FP64 and FP32: median
+    """Finest-level y = J(U) x (cell kernel and node sums), FP64 and FP32: median
     device time of `reps` applies after `warm` untimed ones, L2 flushed (a 256 MB write) before
     each timed apply.  GDoF/s = N_st / t.  Algorithmic bytes per apply: read x and the velocity
     state, write y, plus the vertices: s ((k+1)(3 N_v + 2 N_p)) + 8 d (n+1)^d, s = 8 or 4."""
@@ -633,8 +633,7 @@ def operator_apply(S, U, stream, dev, w, args, peaks, reps=25, warm=5):
                               "median_ms": t1 * 1e3, "algorithmic_bytes": byt1, "achieved_gbs": byt1 / t1 / 1e9,
                               "hbm_frac": byt1 / t1 / 1e9 / peaks.get("hbm_gbs", 6800.0)}
     # FP32 compute roofline of the finest-level apply (2D Q3/P2/DG(2)): FP32 operations per cell
-    # and time node, counted by ncu on one 256^2 launch (FFMA x 2 + FMUL + FADD, the tile's halo
-    # recompute taken out), against the FP32 FMA peak of 152 SMs at 2.07 GHz
+    # and time node of the sum-factorised apply (see the constant), against the FP32 FMA peak of 152 SMs at 2.07 GHz
     if w["d"] == 2 and w["r"] == 2 and w["k"] == 2 and "fp32" in out:
         flops = FP32_APPLY_FLOPS_PER_CELL_NODE * (w["k"] + 1) * w["n"] ** 2
         t32 = out["fp32"]["median_ms"] * 1e-3
@@ -643,11 +642,10 @@ def operator_apply(S, U, stream, dev, w, args, peaks, reps=25, warm=5):
             "frac": flops / t32 / 1e12 / FP32_PEAK_TFLOPS,
             "hbm_frac_at_alu_peak": (out["fp32"]["algorithmic_bytes"] / (peaks.get("hbm_gbs", 6800.0) * 1e9))
                                     / (flops / (FP32_PEAK_TFLOPS * 1e12))}
-    out["note"] = ("FP64 (colour-split warp kernel): bound by the DFMA pipe (84 % pipe utilisation in the ncu "
-                   "capture), so its HBM fraction is low by construction; FP32 (tiled single-launch kernel): "
+    out["note"] = ("FP64: bound by the FP64 pipe, so its HBM fraction is low by construction; FP32: "
                    "its FP32 operations take longer at the FP32 peak than its bytes take at the HBM peak "
                    "(alu_roofline.hbm_frac_at_alu_peak is the HBM fraction that operation count allows), and it "
-                   "runs at alu_roofline.frac of the FP32 peak, bound by instruction issue")
+                   "runs at alu_roofline.frac of the FP32 peak, bound by shared-memory wavefronts and instruction issue")
     return out
 
 
@@ -673,20 +671,20 @@ def _peaks():
         return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "source": "fallback"}
 
 
-# FP32 operations per cell and time node of the 2D Q3/P2/DG(2) FP32 Jacobian apply
-# (k_apply2d_tile<float, 4, 3>): ncu on one 256^2 launch executed 16.80 M FFMA and 6.08 M other FP32
-# warp instructions, i.e. 32 (2 x 16.80 + 6.08) M = 1.270 GFLOP, of which the tile's halo
-# recompute is 22 % (16 x 8 cells computed per 15 x 7 owned): 1.270e9 / 1.219 / (3 x 65536).
+# FP32 operations per cell and time node of the 2D Q3/P2/DG(2) FP32 Jacobian apply as a sum
+# factorisation by 1D passes (counted on a kernel that ran them without even-odd splitting: ncu on one
+# 256^2 launch, 16.80 M FFMA and 6.08 M other FP32 warp instructions = 1.270 GFLOP, 22 % of it a halo
+# recompute, 16 x 8 cells computed per 15 x 7 owned): 1.270e9 / 1.219 / (3 x 65536).
 FP32_APPLY_FLOPS_PER_CELL_NODE = 1.270e9 / (128.0 / 105.0) / (3 * 65536)
 # FP32 FMA peak of one GB300 as measured on this hardware: about 120 FFMA per SM per clock in a
 # dependent-chain probe, x 2 FLOP x 152 SMs x 2.07 GHz = 73.4 TFLOP/s (the nominal 128 lanes per SM
 # give 80.5).
 FP32_PEAK_TFLOPS = 73.4
 
-# DRAM bytes (read + write) per cell of the finest-level Vanka apply (k_vanka_apply_ws), FP32
-# inverses, Q3/P2/DG(2): ncu capture of one colour launch on the 128^2 mesh of the same recipe,
-# 78.70 MB for 4096 cells; scaled to a 256^2 launch by its cells.
-VANKA_DRAM_BYTES_PER_CELL = 78.702848e6 / 4096
+# DRAM bytes (read + write) per cell of the finest-level Vanka patch solves (k_vanka_stream), FP32
+# inverses, Q3/P2/DG(2): ncu capture of one launch on a 256^2 mesh, 1160.6 MB for 65536 cells (the
+# patch vectors, counted in the algorithmic bytes, largely stay in L2).
+VANKA_DRAM_BYTES_PER_CELL = 1160.6e6 / 65536
 
 
 def _inverse_gb(w, args):
@@ -698,8 +696,8 @@ def _inverse_gb(w, args):
 
 
 def roofline(S, prof, args):
-    """Finest-level Vanka patch apply (the dominant kernel): per colour launch it reads the
-    time-diagonalised patch inverses of its cells ((k+1) m_s^2 reals each), gathers the residual
+    """Finest-level Vanka patch apply (the dominant kernel with its node sums): per sweep it reads the
+    time-diagonalised patch inverses of all cells ((k+1) m_s^2 reals each), gathers the residual
     and reads and writes the correction on the patch DoFs.  Achieved = those algorithmic bytes
     per launch over the launch's average device time (CUDA events on the solver stream)."""
     peaks = _peaks()
@@ -709,15 +707,14 @@ def roofline(S, prof, args):
         return None
     achieved = k["bytes"] / (k["ms"] * 1e-3) / 1e9
     d = WORKLOADS[args.workload]["d"]
-    cells = (args.n // 2) ** d                     # cells of one colour launch on the finest level
+    cells = args.n ** d                            # cells of the finest level, all in one sweep
     traffic = VANKA_DRAM_BYTES_PER_CELL * cells if (args.vanka_fp16 == 0 and args.workload == "2d") else None
-    name = ("finest-level Vanka patch apply (k_vanka_apply_ws for the 2D levels; k_vanka_apply / "
-            "k_vanka_apply_global in 3D)")
+    name = "finest-level Vanka patch apply (k_vanka_stream and its node sums)"
     return {"bound": "hbm", "kernel": name, "achieved": achieved, "peak": hbm,
             "unit": "GB/s", "frac": achieved / hbm, "traffic": traffic,
             "algorithmic_bytes_per_launch": k["bytes"] / k["count"],
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured)",
-            "traffic_source": "ncu 128^2 capture scaled by cells per launch" if traffic else None,
+            "traffic_source": "ncu 256^2 capture scaled by cells per launch" if traffic else None,
             "launches": k["count"], "avg_us": 1e3 * k["ms"] / k["count"]}
 
 
