@@ -284,8 +284,7 @@ cudaError_t coarse_invert(const double* A, double* Ainv, double* work, double* p
 // FP64 on few SMs is slow, so small systems are spread over n / 8 blocks (n = 126: 10.2 -> 3.7 us).
 template <typename T, int STEP>
 __global__ void __launch_bounds__(256) k_coarse_mv(const double* A, int n, int nc, const T* b, const double* x1,
-                                                   const double* r,
-                                                   double* __restrict__ y, T* __restrict__ out) {
+                                                   const double* r, double* y, T* out) {
   chain_begin();
   __shared__ double part[32][9];
   A += (int64_t)blockIdx.y * n * n;                   // blockIdx.y: independent slot

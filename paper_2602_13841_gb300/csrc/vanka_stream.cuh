@@ -122,7 +122,7 @@ __device__ __forceinline__ void use_batch(const ChunkBatch<C, U>& c, const T* r,
 template <typename T, typename SI, int D, int N, int KP1>
 __global__ void __launch_bounds__(StreamShape<T, SI, D, N>::THREADS, StreamShape<T, SI, D, N>::BLOCKS)
 k_vanka_stream(LevelArgs<T> L, const SI* inv, const float* scale, const T* res,
-               T* __restrict__ d, T omega_p, const __grid_constant__ TEig<T> te, CellBuf<T> cb, int64_t c0,
+               T* d, T omega_p, const __grid_constant__ TEig<T> te, CellBuf<T> cb, int64_t c0,
                SlotStrides zs, int first, int stream) {
   chain_begin();
   using Sh = StreamShape<T, SI, D, N>;

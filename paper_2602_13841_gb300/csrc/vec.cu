@@ -15,7 +15,7 @@ static inline int grid_for(int64_t n) {
 }
 
 template <typename T>
-__global__ void k_axpby(int64_t n, T a, const T* x, T b, T* __restrict__ y) {
+__global__ void k_axpby(int64_t n, T a, const T* x, T b, T* y) {
   chain_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = a * x[i] + b * y[i];
@@ -29,7 +29,7 @@ cudaError_t vaxpby(int64_t n, T a, const T* x, T b, T* y, cudaStream_t s) {
 }
 
 template <typename S, typename T>
-__global__ void k_copy(int64_t n, const S* x, T* __restrict__ y) {
+__global__ void k_copy(int64_t n, const S* x, T* y) {
   chain_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = (T)x[i];
@@ -88,7 +88,7 @@ __device__ __forceinline__ bool last_block(unsigned* count) {
 
 template <typename T>
 __global__ void k_dots(int64_t n, int m, const T* X, int64_t ldx, const T* w, double* part,
-                       double* __restrict__ out, unsigned* count) {
+                       double* out, unsigned* count) {
   chain_begin();
   __shared__ double red[DOTS_PER_ROW][RED_THREADS];
   const int l0 = blockIdx.y * DOTS_PER_ROW;
@@ -144,7 +144,7 @@ cudaError_t vdots(int64_t n, int m, const T* X, int64_t ldx, const T* w, double*
 // w -= sum_l h[l] X[l]; NORM: also out = sum_i w_i^2 of the result (the same two-stage sum).
 template <typename T, bool NORM>
 __global__ void k_sub_comb(int64_t n, int m, const T* X, int64_t ldx, const double* h,
-                           T* __restrict__ w, double* part, double* __restrict__ out, unsigned* count) {
+                           T* w, double* part, double* out, unsigned* count) {
   chain_begin();
   __shared__ double hs[64];
   __shared__ double red[1][RED_THREADS];
@@ -193,7 +193,7 @@ cudaError_t vsub_comb_norm(int64_t n, int m, const T* X, int64_t ldx, const doub
 struct Coef64 { double v[64]; };
 
 __global__ void k_add_comb(int64_t n, int m, const double* Z, int64_t ldz, Coef64 y,
-                           double* __restrict__ x) {
+                           double* x) {
   chain_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     double acc = x[i];
@@ -214,7 +214,7 @@ cudaError_t vadd_comb_host(int64_t n, int m, const double* Z, int64_t ldz, const
 }
 
 template <typename T>
-__global__ void k_scale_inv_dev(int64_t n, const T* x, const double* nrm, T* __restrict__ y) {
+__global__ void k_scale_inv_dev(int64_t n, const T* x, const double* nrm, T* y) {
   chain_begin();
   const double f = 1.0 / *nrm;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -229,7 +229,7 @@ cudaError_t vscale_inv_dev(int64_t n, const T* x, const double* nrm, T* y, cudaS
 }
 
 template <typename T>
-__global__ void k_scale(int64_t n, T a, const T* x, T* __restrict__ y) {
+__global__ void k_scale(int64_t n, T a, const T* x, T* y) {
   chain_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = a * x[i];
