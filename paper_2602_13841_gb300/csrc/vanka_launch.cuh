@@ -195,7 +195,7 @@ static cudaError_t apply_stream(const Level& lv, const Problem& pb, const SI* in
       const int z1 = z0 + step < lv.n ? z0 + step : lv.n;
       launch_chained(kern, dim3((unsigned)((z1 - z0) * cplane), nb), Sh::THREADS, 0, s,
                      L, inv + b0 * zs.inv, scale ? scale + b0 * zs.scale : nullptr, rb, db, (T)omega_p, te, cb, z0 * cplane, zs, first,
-          stream);
+          stream, wstat);
       note_launch();
       launch_node_sum<T, D, N>(lv, cb, first ? nullptr : db, db, (T)omega, zs.vec, z0, z1, nb, wstat, s);
     }
