@@ -14,14 +14,15 @@ namespace stmg {
 template <typename T>
 cudaError_t MG<T>::allocate(Handle* hh, int slots) {
   h = hh;
-  B = slots < 1 ? 1 : slots;
+  const bool shared = slots > 0;
+  B = shared ? slots : 1;
   nl = (int)h->levels.size();
   U.resize(nl); r.resize(nl); z.resize(nl); t.resize(nl); q.resize(nl); inv.assign(nl, nullptr);
   invh.assign(nl, nullptr); iscale.assign(nl, nullptr);
   inv_slot.assign(nl, 0); invh_slot.assign(nl, 0); scale_slot.assign(nl, 0);
   size_t ea = 0, eb = 0, em = 0, nv = 0, wk = 0;
   try {
-    if (B > 1) nub = (T*)h->dalloc(B * sizeof(T));
+    if (shared) nub = (T*)h->dalloc(B * sizeof(T));
     for (int l = 0; l < nl; ++l) {
       const Level& lv = h->levels[l];
       U[l] = (T*)h->dalloc(B * lv.Nst * sizeof(T));
@@ -158,7 +159,7 @@ cudaError_t MG<T>::sweep(int l, const T* rhs, T* d, int nsweeps, bool zero_start
     if (!first) {
       // q = rhs - J d
       h->kbegin(KC_APPLYP);
-      CKE(launch_level_residual<T>(lv, h->pb, rhs, d, U[l], q[l], s, slots, slots > 1 ? nub : nullptr));
+      CKE(launch_level_residual<T>(lv, h->pb, rhs, d, U[l], q[l], s, slots, nub));
       h->kend(KC_APPLYP);
       res = q[l];
     }
@@ -192,7 +193,7 @@ cudaError_t MG<T>::vcycle_level(int l, const T* rhs, T* d, int slots) {
   else CKE(cudaMemsetAsync(d, 0, (size_t)slots * lv.Nst * sizeof(T), s));
   // t = rhs - J d ; r_{l+1} = P^T t
   h->kbegin(KC_APPLYP);
-  CKE(launch_level_residual<T>(lv, h->pb, rhs, d, U[l], t[l], s, slots, slots > 1 ? nub : nullptr));
+  CKE(launch_level_residual<T>(lv, h->pb, rhs, d, U[l], t[l], s, slots, nub));
   h->kend(KC_APPLYP);
   CKE(tr[l].template restrict_<T>(t[l], r[l + 1], s, slots));
   CKE(vcycle_level(l + 1, r[l + 1], z[l + 1], slots));

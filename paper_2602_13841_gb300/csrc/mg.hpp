@@ -22,7 +22,8 @@ struct MG {
   int nl = 0;
   // Slots: B independent solves of the same level shapes share this hierarchy and are carried
   // through one V-cycle by the same launches (slot j's vectors at j * n_st of each level, its patch
-  // inverses and coarse factors at slot strides); nub holds each slot's viscosity (device, B > 1).
+  // inverses and coarse factors at slot strides); nub holds each slot's viscosity (device; null in a
+  // hierarchy of one handle's own, whose level residuals take the handle's).
   int B = 1;
   T* nub = nullptr;
   std::vector<int64_t> inv_slot, invh_slot, scale_slot;   // per level: slot strides of the patch data
@@ -60,7 +61,7 @@ struct MG {
   cudaError_t vcycle_graph(int slots = 1);   // z[0] = B^{-1} r[0] through the captured graph
   void collect_graph_timers();       // after a stream synchronisation following a replay
 
-  cudaError_t allocate(Handle* h, int slots = 1);
+  cudaError_t allocate(Handle* h, int slots = 0);   // slots: of a group; 0: one handle's own hierarchy
   // Level states from the fine FP64 slab state, patch inverses on every smoothed level,
   // coarse factorisation, for one slot (physics pb; the handle's when null).  Returns
   // cudaErrorUnknown if a patch has a zero pivot.
