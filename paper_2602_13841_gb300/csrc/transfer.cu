@@ -182,6 +182,7 @@ __global__ void k_transfer(const __grid_constant__ TransferArgs<T> A) {
 #pragma unroll 2
         for (int x = 0; x < w[0].y; ++x) {
           const T f = wyz * v[0][x];
+          if (f == (T)0) continue;                    // a gap in the row: its entry does not count, whatever it is
 #pragma unroll
           for (int b = 0; b < MAXKP1; ++b)
             if (b < A.kin) acc[b] += f * s[b * A.vin + x];
