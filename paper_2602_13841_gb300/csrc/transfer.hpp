@@ -16,10 +16,15 @@
 
 namespace stmg {
 
-// A 1D operator: row i combines the win[i].y columns from win[i].x on, with val[i * width + ...].
+// A 1D operator: row i combines columns of the window win[i] = (first, length).  FP32 values: the whole
+// window, val32[i * width + column - first], zero where the row has no entry; FP64: its cnt[i] entries,
+// val64[i * entries + e] at column first + off[i * entries + e].
 struct Line1D {
-  int rows = 0, cols = 0, width = 0;
+  int rows = 0, cols = 0, width = 0, entries = 0;
+  int span = 0;            // columns that the rows of a tile cover together, at most
+  bool gaps = false;       // some window holds zeros
   int2* win = nullptr;     // device
+  int *cnt = nullptr, *off = nullptr;
   double* val64 = nullptr;
   float* val32 = nullptr;
 };
