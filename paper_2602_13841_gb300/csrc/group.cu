@@ -186,7 +186,7 @@ stmg_status stmg_group_create(const stmg_params* p, const double* vertices, int 
     return STMG_ERR_CUDA;
   }
   stmg_handle* hh = nullptr;
-  stmg_status st = stmg_create(p, vertices, reinterpret_cast<stmg_stream>(g->stream), &hh);
+  stmg_status st = create_handle(p, vertices, reinterpret_cast<stmg_stream>(g->stream), slots, &hh);
   if (st != STMG_OK) return st;
   g->core = reinterpret_cast<Handle*>(hh);
   g->B = slots;

@@ -105,4 +105,7 @@ struct Handle {
   bool precond_fp32() const { return prm.precond_precision == STMG_FP32; }
 };
 
+// stmg_create with work space for `slots` columns in one launch (the hierarchy of a group).
+stmg_status create_handle(const stmg_params* p, const double* vertices, stmg_stream stream, int slots, stmg_handle** out);
+
 }  // namespace stmg

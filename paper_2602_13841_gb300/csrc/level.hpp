@@ -60,14 +60,19 @@ cudaError_t launch_level_residual(const Level& lv, const Problem& pb, const T* r
 
 // Bytes of the cell buffer that the operator calls of a level use at most: one column of cell-wise FP64
 // results, capped at 1 GiB (larger meshes run in chunks of cell planes; two planes at least), and
-// at least 16 MiB, so that the batched applies of small levels share launches.
-inline size_t cellbuf_need(int d, int n, int r, int k) {
+// at least 16 MiB, so that the batched applies of small levels share launches.  A group's hierarchy takes its
+// level residuals and sweeps for all slots at once: `slots` columns of es-byte results, each capped alike
+// (1 to 2 % of a slot's patch inverses).
+inline size_t cellbuf_need(int d, int n, int r, int k, int slots = 1, int es = 8) {
   double plane = 8.0 * (k + 1) * d, cells = 1;
   for (int l = 0; l < d; ++l) plane *= r + 2;
   for (int l = 0; l + 1 < d; ++l) cells *= n;
   plane *= cells;
+  const double cap = plane * 2 > 1073741824.0 ? plane * 2 : 1073741824.0;
   double b = plane * n;
-  if (b > 1073741824.0) b = plane * 2 > 1073741824.0 ? plane * 2 : 1073741824.0;
+  const double batch = slots * (b * es / 8.0 < cap ? b * es / 8.0 : cap);
+  if (b > cap) b = cap;
+  if (b < batch) b = batch;
   return (size_t)(b < 16777216.0 ? 16777216.0 : b);
 }
 

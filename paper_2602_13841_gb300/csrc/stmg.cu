@@ -225,6 +225,13 @@ stmg_status stmg_set_physics(stmg_handle* hh, double nu, double tau, int problem
 
 stmg_status stmg_create(const stmg_params* p, const double* vertices, stmg_stream stream,
                         stmg_handle** out) {
+  return create_handle(p, vertices, stream, 1, out);
+}
+
+}  // extern "C"
+
+stmg_status stmg::create_handle(const stmg_params* p, const double* vertices, stmg_stream stream, int slots,
+                                stmg_handle** out) {
   if (!p || !out) return STMG_ERR_ARG;
   *out = nullptr;
   if (p->dim < 2 || p->dim > 3 || p->r < 1 || p->r > 3 || p->k < 0 || p->k > 2 ||
@@ -280,7 +287,8 @@ stmg_status stmg_create(const stmg_params* p, const double* vertices, stmg_strea
       h->levels.push_back(lv);
     }
     size_t cbytes = 0;
-    for (const Level& lv : h->levels) cbytes = std::max(cbytes, cellbuf_need(lv.d, lv.n, lv.r, lv.k));
+    const int es = h->precond_fp32() ? 4 : 8;
+    for (const Level& lv : h->levels) cbytes = std::max(cbytes, cellbuf_need(lv.d, lv.n, lv.r, lv.k, slots, es));
     void* cbuf = h->dalloc(cbytes);
     for (Level& lv : h->levels) { lv.cellbuf = cbuf; lv.cellbuf_bytes = cbytes; }
   } catch (const std::bad_alloc&) {
@@ -296,6 +304,8 @@ stmg_status stmg_create(const stmg_params* p, const double* vertices, stmg_strea
   *out = reinterpret_cast<stmg_handle*>(h.release());
   return STMG_OK;
 }
+
+extern "C" {
 
 long long stmg_launch_count(void) { return launch_count(); }
 
