@@ -261,6 +261,13 @@ stmg_status stmg_set_timing(stmg_handle* h, int on);
  * counterpart in the paper). */
 stmg_status stmg_test_wait_timeout(stmg_handle* h, int on);
 
+/* Test hook of the operator's and the sweeps' work space: cell-wise results are kept in a buffer of the
+ * handle, and levels whose results exceed it run in chunks of cell planes, batched calls in several
+ * passes, with the same results.  From now on the calls of this handle, and of the group that it is attached
+ * to, use at most `bytes` of the buffer (two cell planes of one column at least, else they return
+ * STMG_ERR_CUDA); 0: all of it.  No solve of the group may be running.  Not part of the method. */
+stmg_status stmg_test_cell_buffer(stmg_handle* h, uint64_t bytes);
+
 /* Restrict the per-kernel-class timers of stmg_set_timing to the classes whose bit is set in
  * mask (bit c = class c of stmg_kernel_profile; default: all).  Every timed launch adds two
  * event records (graph nodes inside the captured V-cycle), so timing one class perturbs the

@@ -137,6 +137,8 @@ MG<float>* group_core_mg<float>(Handle* h) { return h->group->core->mg32.get(); 
 template <>
 MG<double>* group_core_mg<double>(Handle* h) { return h->group->core->mg64.get(); }
 
+Handle* group_core(Handle* h) { return h->group->core; }
+
 void group_forget(Handle* h) {
   if (!h->group) return;
   Group& g = *h->group;

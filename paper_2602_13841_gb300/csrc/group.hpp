@@ -19,6 +19,8 @@ void group_forget(Handle* h);
 // A slab solve of h starts / ends (the group waits for the handles inside a solve).
 void group_enter(Handle* h);
 void group_leave(Handle* h);
+// The handle that holds the levels of h's group.
+Handle* group_core(Handle* h);
 // The group's hierarchy (the MG of h's group, of h's preconditioner precision).
 template <typename T>
 MG<T>* group_core_mg(Handle* h);

@@ -45,6 +45,7 @@ struct Handle {
   Problem pb{};
   std::vector<Level> levels;
   std::vector<void*> allocs;
+  size_t cellbuf_bytes = 0;           // of the levels' cell buffer (Level::cellbuf) as allocated
   std::string err;
   // preconditioner (one of the two, by prm.precond_precision)
   std::unique_ptr<MG<float>> mg32;

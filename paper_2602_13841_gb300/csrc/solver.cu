@@ -498,6 +498,21 @@ stmg_status stmg_test_wait_timeout(stmg_handle* hh, int on) {
   return STMG_OK;
 }
 
+static void limit_cellbuf(Handle* h, uint64_t bytes) {
+  for (Level& lv : h->levels) lv.cellbuf_bytes = bytes > 0 && bytes < h->cellbuf_bytes ? (size_t)bytes : h->cellbuf_bytes;
+  // captured V-cycles hold the chunks of the old size
+  if (h->mg32) h->mg32->drop_graph();
+  if (h->mg64) h->mg64->drop_graph();
+}
+
+stmg_status stmg_test_cell_buffer(stmg_handle* hh, uint64_t bytes) {
+  if (!hh) return STMG_ERR_ARG;
+  Handle* h = H(hh);
+  limit_cellbuf(h, bytes);
+  if (h->group) limit_cellbuf(group_core(h), bytes);
+  return STMG_OK;
+}
+
 stmg_status stmg_set_timing_classes(stmg_handle* hh, unsigned mask) {
   if (!hh) return STMG_ERR_ARG;
   H(hh)->kmask = mask;

@@ -290,6 +290,7 @@ stmg_status stmg::create_handle(const stmg_params* p, const double* vertices, st
     const int es = h->precond_fp32() ? 4 : 8;
     for (const Level& lv : h->levels) cbytes = std::max(cbytes, cellbuf_need(lv.d, lv.n, lv.r, lv.k, slots, es));
     void* cbuf = h->dalloc(cbytes);
+    h->cellbuf_bytes = cbytes;
     for (Level& lv : h->levels) { lv.cellbuf = cbuf; lv.cellbuf_bytes = cbytes; }
   } catch (const std::bad_alloc&) {
     return STMG_ERR_OOM;
