@@ -2,9 +2,9 @@
 // kernels of a few microseconds, each reading what the one before wrote, so the time between two of
 // them counts.  A chained kernel may be scheduled while its predecessor's last blocks run: its first
 // statement, chain_begin(), waits until that grid has ended and its writes are visible, then lets the
-// next one be scheduled.  Nothing is read or written before it, so every order of a plain launch holds: a
+// next one be scheduled (the operator's kernels of one time node do so at their end).  Nothing is read or written before it, so every order of a plain launch holds: a
 // grid ends only after its own wait, hence after all grids before it.  A predecessor without
-// chain_begin(), a copy, a memset or an event wait is ordered as by a plain launch; a chained launch
+// a wait, a copy, a memset or an event wait is ordered as by a plain launch; a chained launch
 // captures into a graph like a plain one.  No pointer of a chained kernel is declared __restrict__, const
 // or not: the compiler may take it that the wait does not change what such a pointer points to, and move
 // loads above it.
@@ -17,12 +17,17 @@
 
 namespace stmg {
 
+// chain_wait() opens a chained kernel; chain_release() lets the next one be scheduled once every block has
+// called it (or ended).  Right after the wait (chain_begin) the next kernel's blocks come early, late in the
+// kernel they do not take room from blocks of this grid that have yet to start.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_begin() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  chain_wait();
+  chain_release();
 }
 
-// Launch a kernel that opens with chain_begin(), chained or plainly.  An error is left for cudaGetLastError.
+// Launch a kernel that opens with chain_wait() or chain_begin(), chained or plainly.  An error is left for cudaGetLastError.
 template <typename... P, typename... A>
 static void launch_if_chained(bool chained, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                               A&&... args) {

@@ -63,10 +63,15 @@ static bool plan_cellbuf(const Level& lv, int batch, CellBuf<T>& cb, int64_t& co
 // than the gap it saves; grids of up to a block or two per SM and those of many waves gain (2D, in a graph,
 // chained / plain: FP32 Q2/P1 DG(0) 32^2 7.1 / 7.7 us, 192^2 11.4 / 10.1; Q3/P2 DG(0) 128^2 11.6 / 10.3; Q3/P2
 // DG(2) 96^2 13.9 / 12.7, 256^2 50.6 / 51.0; FP64 Q2/P1 DG(1) 8^2 26.2 / 26.7, 64^2 39.2 / 36.1; Q3/P2 DG(2) 32^2
-// 49.0 / 39.7, 256^2 865 / 866).  3D FP64: few long waves, 16^3 Q3/P2 DG(2) residual 745 / 727 us.
+// 49.0 / 39.7, 256^2 865 / 866).  3D FP64: few long waves, 16^3 Q3/P2 DG(2) residual 745 / 727 us.  The lines are
+// where these measurements put them: no one property of the grids (blocks, waves, time of a block) explains
+// them all.  2D FP32 calls of one time node are always chained, with a late release: by blocks / so, Q2/P1
+// DG(0) 64^2 8.3 / 7.6 us, 128^2 8.9 / 7.9, 192^2 10.9 / 9.9, 256^2 15.8 / 14.9, 512^2 41.0 / 40.7; Q3/P2 DG(0) 128^2
+// 11.1 / 10.2 (three time nodes do worse so: 256^2 Q3/P2 DG(2) 51.2 / 54.7).
 template <typename T, int D>
-static bool chained_cells(int64_t blocks) {
+static bool chained_cells(int64_t blocks, int kp1) {
   constexpr int64_t sms = 152;
+  if (chain_late<T, D>(kp1)) return true;
   if (sizeof(T) == 8) return D == 2 && blocks <= sms;
   return blocks <= 2 * sms || blocks >= 20 * sms;
 }
@@ -127,7 +132,7 @@ static cudaError_t launch_dn(const Level& lv, const Problem& pb, double t0, cons
       }
       const int threads = (cpb * kp1 * TPG + 31) / 32 * 32;
       const int64_t blocks = (c1 - c0 + cpb - 1) / cpb;
-      const bool chained = chained_cells<T, D>(blocks * nb);
+      const bool chained = chained_cells<T, D>(blocks * nb, kp1);
       launch_if_chained(chained, kern, dim3((unsigned)blocks, nb), threads, smem, stream, A, tb,
                      cb, c0, c1, cpb, rb);
       note_launch();

@@ -35,7 +35,8 @@
 //   2D 8^2 Q2/P1 DG(1) FP64 apply    133 -> 35 us
 // and, 2D FP32, against one kernel with a thread per cell on a tile of 16 x 8 cells in shared memory:
 //   256^2 Q3/P2 DG(2) 104 -> 51 us, Q2/P1 DG(1) 28.6 -> 22.7 us; 32^2 59 -> 8.8 us and 14.5 -> 8.0 us
-//   (Q2/P1 DG(0) alone is level: 14.1 -> 15.0 us at 256^2, 8.3 -> 8.2 us at 128^2)
+//   (Q2/P1 DG(0) is the exception: 8.1 -> 7.6 us at 64^2, 8.5 -> 7.9 at 128^2, 13.8 -> 12.8 at 224^2 and level
+//   from 320^2 on, but 8.4 -> 8.9 at 160^2, 9.05 -> 9.9 at 192^2 and 14.3 -> 14.9 at 256^2)
 #pragma once
 #include <type_traits>
 
@@ -43,6 +44,10 @@
 #include "common.cuh"
 
 namespace stmg {
+
+// 2D FP32 calls of one time node release their successor late (see chain.cuh): their grids are short, so that
+// both the gap to the next launch and the blocks that an early successor displaces count.
+template <typename T, int D> __host__ __device__ constexpr bool chain_late(int kp1) { return D == 2 && sizeof(T) == 4 && kp1 == 1; }
 
 enum { MJ = 0, MR = 1, MM = 2 };   // Jacobian apply, residual, mass (w_a M_h, w_a M_p)
 
@@ -1039,7 +1044,9 @@ __device__ __forceinline__ void face2d(const OpArgs<T>& A, const Tab<T>& tb, con
 template <typename T, int N, int MODE, int BT, int MINB>
 __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_constant__ Tab<T> tb, CellBuf<T> cb,
                                                       int64_t c0, int64_t c1, int cpb, const T* rhs) {
-  chain_begin();
+  chain_wait();
+  const bool late = chain_late<T, 2>(tb.k + 1);
+  if (!late) chain_release();
   constexpr bool RES = MODE == MR, MASS = MODE == MM, JAC = MODE == MJ;
   constexpr int Q = N * N, NPC = npress<2, N>();
   constexpr int GS = group2<N>();
@@ -1163,13 +1170,21 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
       for (int c = 0; c < 2; ++c)
 #pragma unroll
         for (int i = 0; i < N; ++i) z[c][i] = RES ? -tb.C[a] * sq[c][i] : (T)0;
-      for (int b = 0; b < kp1; ++b) {
-        const T kab = tb.K[a][b];
-        const T* s = B0 + (b - a) * GS + N * u;
+      if (kp1 == 1) {                                 // the thread's own line
+        const T k00 = tb.K[0][0];
 #pragma unroll
         for (int c = 0; c < 2; ++c)
 #pragma unroll
-          for (int i = 0; i < N; ++i) z[c][i] += kab * s[c * Q + i];
+          for (int i = 0; i < N; ++i) z[c][i] += k00 * xq[c][i];
+      } else {
+        for (int b = 0; b < kp1; ++b) {
+          const T kab = tb.K[a][b];
+          const T* s = B0 + (b - a) * GS + N * u;
+#pragma unroll
+          for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int i = 0; i < N; ++i) z[c][i] += kab * s[c * Q + i];
+        }
       }
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
@@ -1314,6 +1329,7 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
         for (int c = 0; c < 2; ++c) line_ld<T, N>(S + c * Q + u, N, z[c]);
     }
   }
+  if (late) chain_release();
   if (on) {
     const int64_t row = (int64_t)L.n * N;
     T* o = cb.s + blockIdx.y * cb.col + (int64_t)(cc[1] % cb.P) * cb.plane + (int64_t)cc[0] * N + u;
@@ -1346,7 +1362,9 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
 template <typename T, int D, int N, int KP1>
 __global__ void k_node_sum(CellBuf<T> cb, const T* src, T* y, T alpha, int n, int N1, int64_t nnodes, int64_t Nv,
                            int64_t ys, int g0, int64_t count, const int* skip) {
-  chain_begin();
+  chain_wait();
+  constexpr bool late = chain_late<T, D>(KP1);
+  if (!late) chain_release();
   const bool held = skip && *skip;
   if (held && src == y) return;
   y += blockIdx.y * ys;
@@ -1398,6 +1416,7 @@ __global__ void k_node_sum(CellBuf<T> cb, const T* src, T* y, T alpha, int n, in
     for (int ac = 0; ac < KP1 * D; ++ac)
       y[(int64_t)(ac / D) * Nv + (int64_t)(ac % D) * nnodes + node] = held ? old[ac] : old[ac] + alpha * v[ac];
   }
+  if (late) chain_release();
 }
 
 // Face table (FP64) of a 2D level, one thread per boundary face: see OpArgs::fgeo.  With it the longest

@@ -10,7 +10,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 
 def chained_kernels():
-    """{name: parameter list} of the kernels that call chain_begin()."""
+    """{name: parameter list} of the kernels that wait for the one before (chain_begin, chain_wait)."""
     out = {}
     for path in sorted(glob.glob(os.path.join(CSRC, "*.cu*"))):
         src = re.sub(r"//[^\n]*", "", open(path).read())
@@ -20,8 +20,8 @@ def chained_kernels():
                 depth += {"(": 1, ")": -1}.get(src[i], 0)
                 i += 1
             body = src[i:].lstrip()
-            if body.startswith("{") and "chain_begin()" in body[:body.index("\n}")]:
-                assert body[1:].lstrip().startswith("chain_begin();"), m.group(1)
+            if body.startswith("{") and re.search(r"chain_(begin|wait)\(\)", body[:body.index("\n}")]):
+                assert re.match(r"chain_(begin|wait)\(\);", body[1:].lstrip()), m.group(1)
                 out[m.group(1)] = src[m.end():i - 1]
     return out
 
