@@ -252,7 +252,7 @@ stmg_status stmg_set_timing(stmg_handle* h, int on);
 /* Failure-handling test hook.  With on != 0, every following Vanka sweep of this handle outside
  * a captured V-cycle runs a bounded wait into its limit: the sweep with exact patches (smoother = 2)
  * arms the shared-memory barrier of its patch staging for 16 bytes more than it copies; the sweep with
- * surrogate patches (smoother = 0), whose kernels wait for nothing, is preceded by one block that waits
+ * surrogate patches (smoother = 0), whose kernels wait for nothing, is replaced by one block that waits
  * for bytes never sent; the diagonal sweep (smoother = 1) has no wait and runs as usual.
  * The kernel flags the timeout (the exact-patch kernel waits once more, also bounded), the correction
  * is left as it was (zero with zero_start = 1), and the call returns STMG_ERR_TIMEOUT.  No copy is left in

@@ -79,13 +79,13 @@ static bool chained_cells(int64_t blocks, int kp1) {
 // Node sums of the cell planes z0 .. z1 - 1 (see k_node_sum).
 template <typename T, int D, int N>
 static void launch_node_sum(const Level& lv, const CellBuf<T>& cb, const T* src, T* y, T alpha, int64_t ys, int z0,
-                            int z1, int columns, const int* skip, cudaStream_t s, bool chained = true) {
+                            int z1, int columns, cudaStream_t s, bool chained = true) {
   const int g0 = z0 * (N - 1), g1 = z1 == lv.n ? lv.N1 : z1 * (N - 1);
   const int64_t nodes = (int64_t)(g1 - g0) * (D == 2 ? (int64_t)lv.N1 : (int64_t)lv.N1 * lv.N1);
   const int64_t blocks = (nodes + 127) / 128;
   auto kern = lv.k == 0 ? k_node_sum<T, D, N, 1> : lv.k == 1 ? k_node_sum<T, D, N, 2> : k_node_sum<T, D, N, 3>;
   launch_if_chained(chained, kern, dim3((unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), columns), 128, 0, s,
-                 cb, src, y, alpha, lv.n, lv.N1, lv.nnodes, lv.Nv, ys, g0, nodes, skip);
+                 cb, src, y, alpha, lv.n, lv.N1, lv.nnodes, lv.Nv, ys, g0, nodes);
   note_launch();
 }
 
@@ -136,7 +136,7 @@ static cudaError_t launch_dn(const Level& lv, const Problem& pb, double t0, cons
       launch_if_chained(chained, kern, dim3((unsigned)blocks, nb), threads, smem, stream, A, tb,
                      cb, c0, c1, cpb, rb);
       note_launch();
-      launch_node_sum<T, D, N>(lv, cb, rb, A.y, rhs ? (T)-1 : (T)1, ys, z0, z1, nb, nullptr, stream, chained);
+      launch_node_sum<T, D, N>(lv, cb, rb, A.y, rhs ? (T)-1 : (T)1, ys, z0, z1, nb, stream, chained);
     }
   }
   return cudaGetLastError();

@@ -1357,16 +1357,13 @@ __global__ void __launch_bounds__(BT, MINB) k_cells2d(OpArgs<T> A, const __grid_
 // ---------------------------------------------------------------------------- node sums
 // y (velocity part, node planes g0 .. g1-1 of the last axis) = src + alpha * the sum of the cells'
 // contributions at each node (src null: zero; src may be y).  One thread per node, all components and
-// time nodes; the cells of a node in ascending order.  skip: a set flag leaves y as src gives it (src null:
-// zero).
+// time nodes; the cells of a node in ascending order.
 template <typename T, int D, int N, int KP1>
 __global__ void k_node_sum(CellBuf<T> cb, const T* src, T* y, T alpha, int n, int N1, int64_t nnodes, int64_t Nv,
-                           int64_t ys, int g0, int64_t count, const int* skip) {
+                           int64_t ys, int g0, int64_t count) {
   chain_wait();
   constexpr bool late = chain_late<T, D>(KP1);
   if (!late) chain_release();
-  const bool held = skip && *skip;
-  if (held && src == y) return;
   y += blockIdx.y * ys;
   if (src) src += blockIdx.y * ys;
   const T* s = cb.s + blockIdx.y * cb.col;
@@ -1414,7 +1411,7 @@ __global__ void k_node_sum(CellBuf<T> cb, const T* src, T* y, T alpha, int n, in
     }
 #pragma unroll
     for (int ac = 0; ac < KP1 * D; ++ac)
-      y[(int64_t)(ac / D) * Nv + (int64_t)(ac % D) * nnodes + node] = held ? old[ac] : old[ac] + alpha * v[ac];
+      y[(int64_t)(ac / D) * Nv + (int64_t)(ac % D) * nnodes + node] = old[ac] + alpha * v[ac];
   }
   if (late) chain_release();
 }

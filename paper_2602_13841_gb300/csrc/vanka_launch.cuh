@@ -183,9 +183,12 @@ static cudaError_t apply_stream(const Level& lv, const Problem& pb, const SI* in
   const int pairs = te.cplx[0] + (te.nblk > 1 ? te.cplx[1] : 0);
   if (te.nblk != (kp1 + 1) / 2 || pairs != kp1 / 2) return cudaErrorNotSupported;
   auto kern = kp1 == 1 ? k_vanka_stream<T, SI, D, N, 1> : kp1 == 2 ? k_vanka_stream<T, SI, D, N, 2> : k_vanka_stream<T, SI, D, N, 3>;
-  if (extra_tx) {
+  if (extra_tx) {                                     // a sweep that times out leaves d as it was: the hook alone
+    cudaError_t e = first ? cudaMemsetAsync(d, 0, (size_t)slots * zs.vec * sizeof(T), s) : cudaSuccess;
+    if (e != cudaSuccess) return e;
     k_wait_hook<<<1, 1, 0, s>>>(wstat, extra_tx);
     note_launch();
+    return cudaGetLastError();
   }
   for (int b0 = 0; b0 < slots; b0 += (int)cols) {
     const int nb = slots - b0 < (int)cols ? slots - b0 : (int)cols;
@@ -195,9 +198,9 @@ static cudaError_t apply_stream(const Level& lv, const Problem& pb, const SI* in
       const int z1 = z0 + step < lv.n ? z0 + step : lv.n;
       launch_chained(kern, dim3((unsigned)((z1 - z0) * cplane), nb), Sh::THREADS, 0, s,
                      L, inv + b0 * zs.inv, scale ? scale + b0 * zs.scale : nullptr, rb, db, (T)omega_p, te, cb, z0 * cplane, zs, first,
-          stream, wstat);
+          stream);
       note_launch();
-      launch_node_sum<T, D, N>(lv, cb, first ? nullptr : db, db, (T)omega, zs.vec, z0, z1, nb, wstat, s);
+      launch_node_sum<T, D, N>(lv, cb, first ? nullptr : db, db, (T)omega, zs.vec, z0, z1, nb, s);
     }
   }
   return cudaGetLastError();

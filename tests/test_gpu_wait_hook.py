@@ -1,5 +1,5 @@
 """The failure-test hook stmg_test_wait_timeout, smoother by smoother, without a GPU fault.  Surrogate patches
-(0): a block ahead of the sweep waits for bytes that are never sent.  Exact patches (2): the staging
+(0): a block in place of the sweep waits for bytes that are never sent.  Exact patches (2): the staging
 barrier of every patch expects 16 bytes more than are copied.  Both waits are bounded: the sweep returns
 STMG_ERR_TIMEOUT with the correction as it was (zero when it starts from zero), and the handle then gives
 the sweep of a fresh one.  The diagonal sweep (1) has no wait and is not affected."""
