@@ -73,7 +73,8 @@ __global__ void k_to_rowmajor(const double* __restrict__ A, double* __restrict__
 // pivot and an elimination launch per column; n = 126 (2D): 0.37 ms against 1.0 ms in one block.
 constexpr int kPanel = 8;
 
-// key of a pivot candidate: leading bits of |a|, then the row within `bits` low bits (lower rows win)
+// key of a pivot candidate: leading bits of |a|, then the row in the bits of `low` (lower rows win).  A pivot may
+// miss the largest candidate by a factor of 1 - 2^(b - 20), b the bits of the row numbers (n = 816: 2^-10).
 __device__ __forceinline__ unsigned gj_key(double a, int row, unsigned low) {
   // integer comparisons: the FP64 pipe is what the panel steps wait for
   const unsigned hi = (unsigned)__double2hiint(a) & 0x7fffffffu, lo = (unsigned)__double2loint(a);

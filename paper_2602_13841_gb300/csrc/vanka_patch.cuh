@@ -37,6 +37,7 @@ template <typename T> struct PNum<T, false> {
   __device__ static V inv(V a) { return (T)1 / a; }
   __device__ static V neg(V a) { return -a; }
   __device__ static V mul(V a, V b) { return a * b; }
+  __device__ static V add(V a, V b) { return a + b; }
   __device__ static V fma(V acc, V a, V b) { return acc + a * b; }
   __device__ static V fms(V acc, V a, V b) { return acc - a * b; }
   __device__ static T re(V a) { return a; }
@@ -49,6 +50,7 @@ template <typename T> struct PNum<T, true> {
   __device__ static T mag(V a) { return a.x * a.x + a.y * a.y; }
   __device__ static V inv(V a) { const T d = (T)1 / (a.x * a.x + a.y * a.y); return {a.x * d, -a.y * d}; }
   __device__ static V neg(V a) { return {-a.x, -a.y}; }
+  __device__ static V add(V a, V b) { return {a.x + b.x, a.y + b.y}; }
   __device__ static V mul(V a, V b) { return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
   __device__ static V fma(V c, V a, V b) { return {c.x + a.x * b.x - a.y * b.y, c.y + a.x * b.y + a.y * b.x}; }
   __device__ static V fms(V c, V a, V b) { return {c.x - a.x * b.x + a.y * b.y, c.y - a.x * b.y - a.y * b.x}; }
@@ -57,7 +59,10 @@ template <typename T> struct PNum<T, true> {
 };
 
 // Search key of a candidate pivot: the leading bits of its magnitude, then the row (lower rows win).
-// Zero for magnitudes that are not positive (zeros, NaN).
+// Zero for magnitudes that are not positive (zeros, NaN).  The nine low bits are the row's, so that a pivot may
+// miss the largest candidate by a factor of 1 - 2^-14 in FP32 (of the squared magnitude for complex entries)
+// and 1 - 2^-11 in FP64.  Searching by whole magnitudes takes another exchange of bits per step: the errors of
+// rebuilt sweeps against 64 bits were the same to three digits, the rebuild 1 to 5 % slower.
 __device__ __forceinline__ unsigned pivot_key(float a, int row) {
   return a > 0 ? ((__float_as_uint(a) & ~511u) | (unsigned)(511 - row)) : 0u;
 }
@@ -424,23 +429,22 @@ __device__ __forceinline__ bool patch_blocked_block(const VankaArgs<T>& V, const
       reinterpret_cast<Chunk*>(Rm + q * LD)[x] = reinterpret_cast<const Chunk*>(S + piv[p0 + q] * LD)[x];
     }
     __syncthreads();
-    // update: tiles of 4 rows and two chunks (half a row apart), lanes along the row
+    // update: tiles of 4 rows and two chunks (half a row apart), lanes along the row.  The panel's products are
+    // summed from zero and added to the entry once: summed onto the entry, each of them is rounded at its
+    // size.  The entries are loaded four products before the end, so that the last ones hide the latency (3D 16^3
+    // Q3/P2 DG(1) FP32 rebuild: loaded first 19.3 ms, last 21.9, so 19.15; FP64 8^3 55.2 -> 56.5, the additions).
+    // Error of a rebuilt level's sweep against 64 bits, onto the entry -> from zero: that case 5.0e-7 -> 4.4e-7, FP32
+    // 4^3 5.8e-7 -> 3.2e-7, FP64 8^3 Q2/P1 7.9e-16 -> 6.2e-16 (one column at a time: 4.5e-7, 4.5e-7, 7.5e-16).
     constexpr int TC = LD / (2 * VW), TR = (MS + 3) / 4;
     for (int t = tid; t < TR * TC; t += nt) {
       const int i0 = t / TC * 4, l = t - t / TC * TC;
       const int j0 = l * VW, j1 = LD / 2 + l * VW;
       E acc[4][2][VW];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = i0 + r;
-        const bool keep = i < MS && panel_of[i] != ip;
-        const Chunk a = keep ? *reinterpret_cast<const Chunk*>(S + i * LD + j0) : Chunk{};
-        const Chunk b = keep ? *reinterpret_cast<const Chunk*>(S + i * LD + j1) : Chunk{};
+      for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int x = 0; x < VW; ++x) { acc[r][0][x] = a.v[x]; acc[r][1][x] = b.v[x]; }
-      }
-#pragma unroll 4
-      for (int q = 0; q < nb; ++q) {
+        for (int x = 0; x < VW; ++x) { acc[r][0][x] = E{}; acc[r][1][x] = E{}; }
+      const auto product = [&](int q) {
         E wv[4];
         if constexpr (VW <= 4) {
 #pragma unroll
@@ -459,7 +463,20 @@ __device__ __forceinline__ bool patch_blocked_block(const VankaArgs<T>& V, const
             acc[r][0][x] = O::fma(acc[r][0][x], wv[r], a.v[x]);
             acc[r][1][x] = O::fma(acc[r][1][x], wv[r], b.v[x]);
           }
+      };
+      const int q1 = nb > 4 ? nb - 4 : 0;             // the entries are on their way during the last four
+#pragma unroll 4
+      for (int q = 0; q < q1; ++q) product(q);
+      Chunk old[4][2];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int i = i0 + r;
+        const bool keep = i < MS && panel_of[i] != ip;
+        old[r][0] = keep ? *reinterpret_cast<const Chunk*>(S + i * LD + j0) : Chunk{};
+        old[r][1] = keep ? *reinterpret_cast<const Chunk*>(S + i * LD + j1) : Chunk{};
       }
+#pragma unroll 4
+      for (int q = q1; q < nb; ++q) product(q);
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         const int i = i0 + r;
@@ -473,7 +490,7 @@ __device__ __forceinline__ bool patch_blocked_block(const VankaArgs<T>& V, const
             for (int x = 0; x < VW; ++x) o.v[x] = Wm[(j - p0 + x) * LD + i];
           } else {
 #pragma unroll
-            for (int x = 0; x < VW; ++x) o.v[x] = acc[r][h][x];
+            for (int x = 0; x < VW; ++x) o.v[x] = O::add(old[r][h].v[x], acc[r][h][x]);
           }
           *reinterpret_cast<Chunk*>(S + i * LD + j) = o;
         }
