@@ -16,9 +16,6 @@
 
 namespace stmg {
 
-
-
-
 template <int D, int N>
 static constexpr size_t elem_smem(size_t es) { return es * elem_table_entries<D, N>(); }
 

@@ -242,18 +242,6 @@ cudaError_t vscale(int64_t n, T a, const T* x, T* y, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <typename T>
-__global__ void k_fill(int64_t n, T v, T* __restrict__ x) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) x[i] = v;
-}
-
-template <typename T>
-cudaError_t vfill(int64_t n, T v, T* x, cudaStream_t s) {
-  k_fill<T><<<grid_for(n), 256, 0, s>>>(n, v, x);
-  note_launch();
-  return cudaGetLastError();
-}
-
 __global__ void k_finite(int64_t n, const double* x, int* flag) {
   chain_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -282,7 +270,5 @@ template cudaError_t vscale_inv_dev<double>(int64_t, const double*, const double
 template cudaError_t vscale_inv_dev<float>(int64_t, const float*, const double*, float*, cudaStream_t);
 template cudaError_t vscale<float>(int64_t, float, const float*, float*, cudaStream_t);
 template cudaError_t vscale<double>(int64_t, double, const double*, double*, cudaStream_t);
-template cudaError_t vfill<float>(int64_t, float, float*, cudaStream_t);
-template cudaError_t vfill<double>(int64_t, double, double*, cudaStream_t);
 
 }  // namespace stmg

@@ -38,9 +38,6 @@ cudaError_t vscale_inv_dev(int64_t n, const T* x, const double* nrm, T* y, cudaS
 // y = a * x
 template <typename T>
 cudaError_t vscale(int64_t n, T a, const T* x, T* y, cudaStream_t s);
-// set x[i] = v for i in [0, n)
-template <typename T>
-cudaError_t vfill(int64_t n, T v, T* x, cudaStream_t s);
 // NaN / Inf check: *flag = 1 if any entry of x is not finite
 cudaError_t vfinite(int64_t n, const double* x, int* flag, cudaStream_t s);
 
