@@ -20,7 +20,9 @@
  * otherwise; its element type follows the precision argument (double for STMG_FP64, float
  * for STMG_FP32).  The handle owns meshes, level data, smoother factors and Krylov scratch.
  * Work is enqueued on the handle's stream; a call returns after enqueueing unless it needs a
- * device scalar (norms, Krylov control), in which case it synchronises that stream.
+ * device scalar (norms, Krylov control), in which case it synchronises that stream.  The calls of a handle
+ * share its work space (the operator's cell-wise results among it), so a call captured into a graph is
+ * replayed in order with the handle's other work.
  * Errors: every call returns a stmg_status; stmg_last_error() describes the last failure of a
  * handle.  No C++ exception crosses the ABI.  A handle is used by one host thread at a time;
  * distinct handles are independent.
@@ -274,10 +276,12 @@ stmg_status stmg_test_cell_buffer(stmg_handle* h, uint64_t bytes);
  * solve less than timing all of them; the phase times are recorded either way. */
 stmg_status stmg_set_timing_classes(stmg_handle* h, unsigned mask);
 
-/* Device time (ms), launches and algorithmic bytes accumulated per kernel class while timing is
- * on (collected at the end of each stmg_slab_solve).  Classes: 0 FP64 Jacobian apply (outer
+/* Device time (ms), timed calls and algorithmic bytes accumulated per kernel class while timing is
+ * on (collected at the end of each stmg_slab_solve).  *launches counts the calls timed, whatever the
+ * number of kernels in one: one per operator call and per sweep (two launches each, more in chunks, or
+ * 2^d with smoother = 1 or 2), four per level of a build.  Classes: 0 FP64 Jacobian apply (outer
  * FGMRES), 1 preconditioner-precision Jacobian apply (level residuals), 2 residual, 3 Vanka
- * patch apply (one per sweep; bytes = patch inverses + patch vectors), 4 Vanka build
+ * patch apply (bytes = patch inverses + patch vectors), 4 Vanka build
  * (element matrices, patch assembly and inversion), 5 mass apply, 6 Vanka patch apply on the
  * finest level only (a subset of class 3). */
 stmg_status stmg_kernel_profile(const stmg_handle* h, int cls, double* ms, long long* launches,
@@ -300,7 +304,8 @@ stmg_status stmg_slab_solve(stmg_handle* h, double t_start, const double* V_prev
  * stmg_params except viscosity and problem data, the same vertices).  An attached handle's
  * smoother builds fill its own slot, and each preconditioner application (one per FGMRES
  * iteration) joins the next batched V-cycle of the group: every kernel of the V-cycle chain
- * (level residuals, Vanka sweeps, transfers, coarse solve) is launched once for all ready slots.
+ * (level residuals, Vanka sweeps, transfers, coarse solve) is launched once for all ready slots (levels
+ * of more than 1 GiB of cell-wise results in chunks).
  * Batching is the serving pattern of concurrent same-shape requests; the paper has no
  * counterpart (its solver runs one problem at a time).  A round starts as soon as every attached
  * handle that is inside stmg_slab_solve is waiting, or 200 microseconds after the first one

@@ -27,12 +27,14 @@
 // planes (slot = plane mod P), so meshes beyond its size run in chunks of planes, each chunk
 // finding the previous chunk's last plane still in place.
 //
-// What bounds it: FP64 the FP64 pipe (2 multiply-adds per clock and SM; 84 % busy on 3D Q2/P1), FP32
-// shared-memory wavefronts and instruction issue.  Measured against the colour-by-colour kernels this
+// What bounds it: FP64 the FP64 pipe (2 multiply-adds per clock and SM; 83 % busy in the 3D 24^3 Q2/P1 DG(2)
+// apply, 86 % in the 16^3 Q3/P2 DG(2) residual), FP32 shared-memory wavefronts (a third of them bank conflicts
+// in 2D Q3/P2) and instruction issue.  A 3D boundary cell costs about three interior ones (FP64 residual, Q3/P2
+// DG(2), per cell: 16^3 181 ns, 24^3 149, 40^3 135).  Measured against the colour-by-colour kernels this
 // replaces (a zero fill, then a volume and a face launch per colour with one thread per point):
-//   3D 64^3 Q2/P1 DG(2) FP64 apply 20.14 -> 12.63 ms    3D 37^3 Q3/P2 DG(1) FP32 apply 940 -> 284 us
-//   3D 16^3 Q3/P2 DG(2) residual    3.00 -> 0.73 ms     2D 256^2 Q3/P2 DG(2) FP64 apply 1086 -> 879 us
-//   2D 8^2 Q2/P1 DG(1) FP64 apply    133 -> 35 us
+//   3D 64^3 Q2/P1 DG(2) FP64 apply 20.14 -> 12.64 ms    3D 37^3 Q3/P2 DG(1) FP32 apply 940 -> 279 us
+//   3D 16^3 Q3/P2 DG(2) residual    3.00 -> 0.73 ms     2D 256^2 Q3/P2 DG(2) FP64 apply 1086 -> 870 us
+//   2D 8^2 Q2/P1 DG(1) FP64 apply    133 -> 27 us
 // and, 2D FP32, against one kernel with a thread per cell on a tile of 16 x 8 cells in shared memory:
 //   256^2 Q3/P2 DG(2) 104 -> 51 us, Q2/P1 DG(1) 28.6 -> 22.7 us; 32^2 59 -> 8.8 us and 14.5 -> 8.0 us
 //   (Q2/P1 DG(0) is the exception: 8.1 -> 7.6 us at 64^2, 8.5 -> 7.9 at 128^2, 13.8 -> 12.8 at 224^2 and level
@@ -226,7 +228,7 @@ __device__ __forceinline__ void row_st(T* s, const T (&v)[N]) {
 // that the lines along y of a warp's threads fall into different banks.
 template <int N> __host__ __device__ constexpr int plane3() { return N == 4 ? 20 : N * N; }
 template <int N> __host__ __device__ constexpr int arr3() { return plane3<N>() * N; }
-template <int N> __host__ __device__ constexpr int even4(int e) { return (e + 3) & ~3; }
+__host__ __device__ constexpr int even4(int e) { return (e + 3) & ~3; }
 // Smallest stride >= e that is `want` mod 32: neighbouring groups of a warp, `stride` entries apart, then
 // use different banks for their lines along every axis (with a stride of a multiple of 32 the lines of
 // 2D Q2/P1 collided: 256^2 Q2/P1 DG(2) FP32 apply 88 us instead of 35).
@@ -247,7 +249,7 @@ template <int N> __host__ __device__ constexpr int group2() {
 template <typename T, int N, int MODE>
 __host__ __device__ inline size_t cells3d_smem(int cpb, int kp1) {
   constexpr int QP = arr3<N>(), Q = N * N * N;
-  const size_t cell = even4<N>(10 * Q + 24 + (MODE == MR ? 3 * QP : 0));  // geometry, map, V_{n-1}
+  const size_t cell = even4(10 * Q + 24 + (MODE == MR ? 3 * QP : 0));  // geometry, map, V_{n-1}
   return sizeof(T) * ((size_t)cpb * kp1 * group3<N>() + (size_t)cpb * cell + 2 * MAXN * MAXN + MAXN * 4 + 2 * MAXN);
 }
 template <typename T, int N>
@@ -507,7 +509,7 @@ __global__ void __launch_bounds__(BT, MINB) k_cells3d(OpArgs<T> A, const __grid_
   constexpr bool RES = MODE == MR, MASS = MODE == MM, JAC = MODE == MJ;
   constexpr int NN = N * N, Q = N * NN, PL = plane3<N>(), QP = arr3<N>(), NPC = npress<3, N>();
   constexpr int GS = group3<N>();
-  constexpr int CS = even4<N>(10 * Q + 24 + (RES ? 3 * QP : 0));
+  constexpr int CS = even4(10 * Q + 24 + (RES ? 3 * QP : 0));
   const LevelArgs<T>& L = A.L;
   const int kp1 = tb.k + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -1,7 +1,7 @@
-"""Failure handling on the GPU without a GPU fault: the Vanka apply stages each patch inverse by
-a bulk copy and waits for it on a shared-memory barrier with an iteration limit.  The test hook
-stmg_test_wait_timeout makes that wait run out (the barrier expects bytes that are never sent);
-the sweep must return STMG_ERR_TIMEOUT with its message, and once the hook is off the same handle
+"""Failure handling on the GPU without a GPU fault, for the default smoother: the test hook
+stmg_test_wait_timeout puts a block in place of the sweep that waits, with a limit, for bytes that are never
+sent to its shared-memory barrier (the sweep's own kernels have no wait; the one of the exact patches is
+covered in test_gpu_wait_hook.py).  The sweep must return STMG_ERR_TIMEOUT with its message, and once the hook is off the same handle
 must give the sweep of a fresh handle again (the context stayed usable)."""
 import ctypes
 
